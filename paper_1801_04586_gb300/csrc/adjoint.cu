@@ -288,9 +288,9 @@ __device__ __forceinline__ void force_adj(const ForceArgs &F, const Geom &g, int
     if (FM == kForceUniform) {
         fx = F.fx; fy = F.fy; fz = F.fz;
     } else if (FM == kForceProfileZ) {
-        fx = __ldg(F.profile + z); fy = __ldg(F.profile + g.nz + z); fz = __ldg(F.profile + 2 * g.nz + z);
+        fx = F.profile[z]; fy = F.profile[g.nz + z]; fz = F.profile[2 * g.nz + z];
     } else {
-        fx = __ldg(F.field + self); fy = __ldg(F.field + F.n + self); fz = __ldg(F.field + 2 * F.n + self);
+        fx = F.field[self]; fy = F.field[F.n + self]; fz = F.field[2 * F.n + self];
     }
     fx *= F.scale;
     fy *= F.scale;
@@ -381,9 +381,10 @@ __device__ __forceinline__ void send_adjoint_faces(float *lam, const Geom &g, in
 // SLAB: a z-slab (pull through the halo map, gathers across halo faces from
 // lam_next's receive planes, send planes of lam written).
 template <typename S, int FM, bool WALLS, bool SLAB>
-__global__ void __launch_bounds__(256, 3) k_adjoint_step(const S *__restrict__ state, const float *__restrict__ lam_next,
+__global__ void __launch_bounds__(256, 3) k_adjoint_step(const S *state, const float *lam_next,
                                                       float *__restrict__ lam, float *__restrict__ gF, Geom g,
                                                       Rates r, ForceArgs F, int64_t n) {
+    grid_dependency_wait();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z;
@@ -399,7 +400,7 @@ __global__ void __launch_bounds__(256, 3) k_adjoint_step(const S *__restrict__ s
         else
             push_targets<WALLS>(g, x, y, z, off, pop);
 #pragma unroll
-        for (int i = 0; i < kQ; ++i) l[i] = __ldg(lam_next + (size_t)pop[i] * n + off[i]);
+        for (int i = 0; i < kQ; ++i) l[i] = lam_next[(size_t)pop[i] * n + off[i]];
     }
     float h[kQ];
     uint32_t self;
@@ -426,8 +427,9 @@ __global__ void __launch_bounds__(256, 3) k_adjoint_step(const S *__restrict__ s
 // Seed from a cotangent gu (3 x n) on the Eq. 9 velocity of the state in
 // `state`: lam_i = sum_a gu_a (e_ia - u_a)/rho, gF = gu/(2 rho) (written).
 template <typename S, int FM, bool WALLS, bool SLAB>
-__global__ void k_adjoint_seed(const S *__restrict__ state, const float *__restrict__ gu, float *__restrict__ lam,
+__global__ void k_adjoint_seed(const S *state, const float *gu, float *__restrict__ lam,
                                float *__restrict__ gF, Geom g, ForceArgs F, int64_t n) {
+    grid_dependency_wait();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z;
@@ -463,11 +465,11 @@ __global__ void k_adjoint_seed(const S *__restrict__ state, const float *__restr
 #define CLBM_ADJ_LAUNCH(FMODE, walls, slab, KERNEL, ...)                                                     \
     do {                                                                                                    \
         if (slab) {                                                                                         \
-            if (walls) KERNEL<S, FMODE, true, true><<<L.grid, L.block, 0, L.stream>>>(__VA_ARGS__);         \
-            else KERNEL<S, FMODE, false, true><<<L.grid, L.block, 0, L.stream>>>(__VA_ARGS__);              \
+            if (walls) launch_overlapped(KERNEL<S, FMODE, true, true>, L.grid, L.block, 0, L.stream, L.overlap, __VA_ARGS__);         \
+            else launch_overlapped(KERNEL<S, FMODE, false, true>, L.grid, L.block, 0, L.stream, L.overlap, __VA_ARGS__);              \
         } else {                                                                                            \
-            if (walls) KERNEL<S, FMODE, true, false><<<L.grid, L.block, 0, L.stream>>>(__VA_ARGS__);        \
-            else KERNEL<S, FMODE, false, false><<<L.grid, L.block, 0, L.stream>>>(__VA_ARGS__);             \
+            if (walls) launch_overlapped(KERNEL<S, FMODE, true, false>, L.grid, L.block, 0, L.stream, L.overlap, __VA_ARGS__);        \
+            else launch_overlapped(KERNEL<S, FMODE, false, false>, L.grid, L.block, 0, L.stream, L.overlap, __VA_ARGS__);             \
         }                                                                                                   \
     } while (0)
 

@@ -67,12 +67,13 @@ __device__ __forceinline__ uint32_t pull_node(const S *src, const Geom &g, int x
     int pop[kQ];
     state_slots<WALLS>(g, x, y, z, map, off, pop);
 #pragma unroll
-    for (int i = 0; i < kQ; ++i) h[i] = Codec<S>::load_plain(src + CLBM_IDX(g, (size_t)pop[i] * g.stride + off[i]));
+    for (int i = 0; i < kQ; ++i) h[i] = Codec<S>::load(src + CLBM_IDX(g, (size_t)pop[i] * g.stride + off[i]));
     return ((uint32_t)z * g.ny + y) * g.nx + x;
 }
 
 template <typename S, bool WALLS>
-__global__ void k_scatter(S *dst, Geom g, int map, const float *__restrict__ f, int64_t n, int deviation) {
+__global__ void k_scatter(S *dst, Geom g, int map, const float *f, int64_t n, int deviation) {
+    grid_dependency_wait();
     int x, y, z;
     if (!node_of(g, x, y, z)) return;
     const uint32_t self = ((uint32_t)z * g.ny + y) * g.nx + x;
@@ -86,8 +87,9 @@ __global__ void k_scatter(S *dst, Geom g, int map, const float *__restrict__ f, 
 }
 
 template <typename S, int FM, bool WALLS>
-__global__ void k_init_eq(S *dst, Geom g, int map, const float *__restrict__ rho, const float *__restrict__ u,
+__global__ void k_init_eq(S *dst, Geom g, int map, const float *rho, const float *u,
                           int64_t n, ForceArgs F, int z0) {
+    grid_dependency_wait();
     int x, y, z;
     if (!node_of(g, x, y, z, z0)) return;
     const uint32_t self = ((uint32_t)z * g.ny + y) * g.nx + x;
@@ -105,6 +107,7 @@ __global__ void k_init_eq(S *dst, Geom g, int map, const float *__restrict__ rho
 
 template <typename S, bool WALLS>
 __global__ void k_gather(const S *src, Geom g, int map, float *__restrict__ f, int64_t n, int deviation) {
+    grid_dependency_wait();
     int x, y, z;
     if (!node_of(g, x, y, z)) return;
     float h[kQ];
@@ -116,6 +119,7 @@ __global__ void k_gather(const S *src, Geom g, int map, float *__restrict__ f, i
 template <typename S, int FM, bool WALLS>
 __global__ void k_macros(const S *src, Geom g, int map, ForceArgs F, float *__restrict__ rho,
                          float *__restrict__ u, int64_t n, int z0) {
+    grid_dependency_wait();
     int x, y, z;
     if (!node_of(g, x, y, z, z0)) return;
     float h[kQ];
@@ -182,7 +186,7 @@ __global__ void k_reduce_moments(const S *src, Geom g, int map, ForceArgs F, lon
     block_sum_fixed<4>(q, partials + (size_t)blockIdx.x * 4);
 }
 
-__global__ void k_reduce_pair(const float *__restrict__ a, const float *__restrict__ b, int64_t n,
+__global__ void k_reduce_pair(const float *a, const float *b, int64_t n,
                               double *partials) {
     double v[3] = {0.0, 0.0, 0.0};
     for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < n; s += (int64_t)gridDim.x * blockDim.x) {
@@ -205,7 +209,7 @@ __global__ void k_reduce_pair(const float *__restrict__ a, const float *__restri
 
 template <typename S, bool W>
 static void scatter_t(const Launch &L, void *dst, const float *f, int64_t n, int dev) {
-    k_scatter<S, W><<<L.grid, L.block, 0, L.stream>>>((S *)dst, L.g, L.map, f, n, dev);
+    launch_overlapped(k_scatter<S, W>, L.grid, L.block, 0, L.stream, L.overlap, (S *)dst, L.g, L.map, f, n, dev);
 }
 
 cudaError_t launch_scatter(int storage, const Launch &L, void *dst, const float *f, int64_t n, int deviation) {
@@ -233,8 +237,10 @@ static void init_t(const Launch &L, void *dst, const float *rho, const float *u,
     int z0;
     const dim3 grid = plane_grid(L, z0);
     if (grid.z == 0) return;
-    if (L.g.walls) k_init_eq<S, FM, true><<<grid, L.block, 0, L.stream>>>((S *)dst, L.g, L.map, rho, u, n, F, z0);
-    else k_init_eq<S, FM, false><<<grid, L.block, 0, L.stream>>>((S *)dst, L.g, L.map, rho, u, n, F, z0);
+    if (L.g.walls) launch_overlapped(k_init_eq<S, FM, true>, grid, L.block, 0, L.stream, L.overlap, (S *)dst, L.g,
+                                     L.map, rho, u, n, F, z0);
+    else launch_overlapped(k_init_eq<S, FM, false>, grid, L.block, 0, L.stream, L.overlap, (S *)dst, L.g, L.map, rho,
+                           u, n, F, z0);
 }
 
 cudaError_t launch_init_eq(int storage, const Launch &L, void *dst, const float *rho, const float *u, int64_t n,
@@ -251,8 +257,10 @@ cudaError_t launch_init_eq(int storage, const Launch &L, void *dst, const float 
 
 cudaError_t launch_gather(int storage, const Launch &L, const void *src, float *f, int64_t n, int deviation) {
     CLBM_DISPATCH_STORAGE(storage, {
-        if (L.g.walls) k_gather<S, true><<<L.grid, L.block, 0, L.stream>>>((const S *)src, L.g, L.map, f, n, deviation);
-        else k_gather<S, false><<<L.grid, L.block, 0, L.stream>>>((const S *)src, L.g, L.map, f, n, deviation);
+        if (L.g.walls) launch_overlapped(k_gather<S, true>, L.grid, L.block, 0, L.stream, L.overlap, (const S *)src,
+                                         L.g, L.map, f, n, deviation);
+        else launch_overlapped(k_gather<S, false>, L.grid, L.block, 0, L.stream, L.overlap, (const S *)src, L.g,
+                               L.map, f, n, deviation);
     })
     return cudaGetLastError();
 }
@@ -263,9 +271,11 @@ static void macros_t(const Launch &L, const void *src, const ForceArgs &F, float
     const dim3 grid = plane_grid(L, z0);
     if (grid.z == 0) return;
     if (L.g.walls)
-        k_macros<S, FM, true><<<grid, L.block, 0, L.stream>>>((const S *)src, L.g, L.map, F, rho, u, n, z0);
+        launch_overlapped(k_macros<S, FM, true>, grid, L.block, 0, L.stream, L.overlap, (const S *)src, L.g, L.map,
+                          F, rho, u, n, z0);
     else
-        k_macros<S, FM, false><<<grid, L.block, 0, L.stream>>>((const S *)src, L.g, L.map, F, rho, u, n, z0);
+        launch_overlapped(k_macros<S, FM, false>, grid, L.block, 0, L.stream, L.overlap, (const S *)src, L.g, L.map,
+                          F, rho, u, n, z0);
 }
 
 cudaError_t launch_macros(int storage, const Launch &L, const void *src, const ForceArgs &F, float *rho, float *u,

@@ -41,7 +41,7 @@ __device__ __forceinline__ bool on_wall_face(const Geom &g, int x, int y, int z)
 // bounce-back map alone; on the batched step, whose domains all have walls,
 // 1 % faster.)
 template <typename S, bool WALLS>
-__device__ __forceinline__ uint32_t pull_load(const S *__restrict__ src, const Geom &g, int x, int y, int z,
+__device__ __forceinline__ uint32_t pull_load(const S *src, const Geom &g, int x, int y, int z,
                                               float (&h)[kQ]) {
     uint32_t off[kQ];
     int pop[kQ];
@@ -69,7 +69,7 @@ struct DomainDesc {
 // usual case); otherwise it is read through the read-only cache. The next
 // tile's entry is fetched while the current tile is processed.
 template <typename S, bool SMEM>
-__global__ void __launch_bounds__(512) k_batch_step(const S *__restrict__ A, S *__restrict__ B,
+__global__ void __launch_bounds__(512) k_batch_step(const S *A, S *__restrict__ B,
                                                     const DomainDesc *__restrict__ doms, int ndom,
                                                     const int4 *__restrict__ tiles, int ntiles,
                                                     int *__restrict__ flag) {
@@ -78,6 +78,7 @@ __global__ void __launch_bounds__(512) k_batch_step(const S *__restrict__ A, S *
         for (int i = threadIdx.x; i < ndom; i += blockDim.x) sdom[i] = doms[i];
         __syncthreads();
     }
+    grid_dependency_wait();  // (the domain table and the work list stay unchanged while steps run)
     int t = blockIdx.x;
     if (t >= ntiles) return;
     int4 tile = __ldg(tiles + t);  // (domain, x, y, z) of the tile's first node
@@ -122,6 +123,7 @@ __global__ void __launch_bounds__(512) k_batch_step_aa(S *A, const DomainDesc *_
         for (int i = threadIdx.x; i < ndom; i += blockDim.x) sdom[i] = doms[i];
         __syncthreads();
     }
+    grid_dependency_wait();  // (the domain table and the work list stay unchanged while steps run)
     int t = blockIdx.x;
     if (t >= ntiles) return;
     int4 tile = __ldg(tiles + t);
@@ -170,44 +172,53 @@ constexpr int kSmemDomains = 512;  // domain tables up to this size are staged i
 
 template <typename S>
 static cudaError_t batch_launch_t(const void *A, void *B, const DomainDesc *doms, int ndom, const int4 *tiles,
-                                  int ntiles, int grid, dim3 block, int *flag, cudaStream_t s) {
+                                  int ntiles, int grid, dim3 block, int *flag, cudaStream_t s,
+                                bool overlap) {
     if (ndom <= kSmemDomains)
-        k_batch_step<S, true><<<grid, block, sizeof(DomainDesc) * ndom, s>>>((const S *)A, (S *)B, doms, ndom, tiles,
-                                                                            ntiles, flag);
+        launch_overlapped(k_batch_step<S, true>, grid, block, sizeof(DomainDesc) * ndom, s, overlap, (const S *)A,
+                          (S *)B, doms, ndom, tiles, ntiles, flag);
     else
-        k_batch_step<S, false><<<grid, block, 0, s>>>((const S *)A, (S *)B, doms, ndom, tiles, ntiles, flag);
+        launch_overlapped(k_batch_step<S, false>, grid, block, 0, s, overlap, (const S *)A, (S *)B, doms, ndom,
+                          tiles, ntiles, flag);
     return cudaGetLastError();
 }
 
 template <typename S>
 static cudaError_t batch_launch_aa_t(void *A, const DomainDesc *doms, int ndom, const int4 *tiles, int ntiles,
-                                     int grid, dim3 block, int *flag, cudaStream_t s, bool odd) {
+                                     int grid, dim3 block, int *flag, cudaStream_t s, bool overlap,
+                                   bool odd) {
     const size_t sm = ndom <= kSmemDomains ? sizeof(DomainDesc) * ndom : 0;
     if (ndom <= kSmemDomains) {
-        if (odd) k_batch_step_aa<S, true, true><<<grid, block, sm, s>>>((S *)A, doms, ndom, tiles, ntiles, flag);
-        else k_batch_step_aa<S, true, false><<<grid, block, sm, s>>>((S *)A, doms, ndom, tiles, ntiles, flag);
+        if (odd) launch_overlapped(k_batch_step_aa<S, true, true>, grid, block, sm, s, overlap, (S *)A, doms, ndom,
+                                   tiles, ntiles, flag);
+        else launch_overlapped(k_batch_step_aa<S, true, false>, grid, block, sm, s, overlap, (S *)A, doms, ndom,
+                               tiles, ntiles, flag);
     } else {
-        if (odd) k_batch_step_aa<S, false, true><<<grid, block, 0, s>>>((S *)A, doms, ndom, tiles, ntiles, flag);
-        else k_batch_step_aa<S, false, false><<<grid, block, 0, s>>>((S *)A, doms, ndom, tiles, ntiles, flag);
+        if (odd) launch_overlapped(k_batch_step_aa<S, false, true>, grid, block, 0, s, overlap, (S *)A, doms, ndom,
+                                   tiles, ntiles, flag);
+        else launch_overlapped(k_batch_step_aa<S, false, false>, grid, block, 0, s, overlap, (S *)A, doms, ndom,
+                               tiles, ntiles, flag);
     }
     return cudaGetLastError();
 }
 
 static cudaError_t batch_launch_aa(int storage, void *A, const DomainDesc *doms, int ndom, const int4 *tiles,
-                                   int ntiles, int grid, dim3 block, int *flag, cudaStream_t s, bool odd) {
+                                   int ntiles, int grid, dim3 block, int *flag, cudaStream_t s, bool overlap,
+                                   bool odd) {
     switch (storage) {
-        case 0: return batch_launch_aa_t<float>(A, doms, ndom, tiles, ntiles, grid, block, flag, s, odd);
-        case 1: return batch_launch_aa_t<__half>(A, doms, ndom, tiles, ntiles, grid, block, flag, s, odd);
-        default: return batch_launch_aa_t<__nv_bfloat16>(A, doms, ndom, tiles, ntiles, grid, block, flag, s, odd);
+        case 0: return batch_launch_aa_t<float>(A, doms, ndom, tiles, ntiles, grid, block, flag, s, overlap, odd);
+        case 1: return batch_launch_aa_t<__half>(A, doms, ndom, tiles, ntiles, grid, block, flag, s, overlap, odd);
+        default: return batch_launch_aa_t<__nv_bfloat16>(A, doms, ndom, tiles, ntiles, grid, block, flag, s, overlap, odd);
     }
 }
 
 static cudaError_t batch_launch(int storage, const void *A, void *B, const DomainDesc *doms, int ndom,
-                                const int4 *tiles, int ntiles, int grid, dim3 block, int *flag, cudaStream_t s) {
+                                const int4 *tiles, int ntiles, int grid, dim3 block, int *flag, cudaStream_t s,
+                                bool overlap) {
     switch (storage) {
-        case 0: return batch_launch_t<float>(A, B, doms, ndom, tiles, ntiles, grid, block, flag, s);
-        case 1: return batch_launch_t<__half>(A, B, doms, ndom, tiles, ntiles, grid, block, flag, s);
-        default: return batch_launch_t<__nv_bfloat16>(A, B, doms, ndom, tiles, ntiles, grid, block, flag, s);
+        case 0: return batch_launch_t<float>(A, B, doms, ndom, tiles, ntiles, grid, block, flag, s, overlap);
+        case 1: return batch_launch_t<__half>(A, B, doms, ndom, tiles, ntiles, grid, block, flag, s, overlap);
+        default: return batch_launch_t<__nv_bfloat16>(A, B, doms, ndom, tiles, ntiles, grid, block, flag, s, overlap);
     }
 }
 
@@ -338,11 +349,12 @@ int build_tiles(clbm_batch *b, int T) {
 // One step of every domain: A/B from buffer `from`; in place, the odd kind when
 // `from` is 1 (the parity of the step).
 cudaError_t launch_all(clbm_batch *b, cudaStream_t s, int from) {
+    const bool overlap = s != b->capture_stream;
     if (b->aa)
         return batch_launch_aa(b->storage, b->buf[0], b->d_descs, b->ndom, b->d_tiles, b->ntiles, b->grid, b->block,
-                               b->d_flag, s, from == 1);
+                               b->d_flag, s, overlap, from == 1);
     return batch_launch(b->storage, b->buf[from], b->buf[from ^ 1], b->d_descs, b->ndom, b->d_tiles, b->ntiles,
-                        b->grid, b->block, b->d_flag, s);
+                        b->grid, b->block, b->d_flag, s, overlap);
 }
 
 // Capture graph_steps steps starting from buffer 0 (in place: from an even

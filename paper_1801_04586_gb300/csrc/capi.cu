@@ -238,6 +238,7 @@ int ensure_graph(clbm_ctx *c) {
     }
     Launch L = step_launch_of(c);
     L.stream = c->cap_stream;
+    L.overlap = false;
     cudaGraph_t g = nullptr;
     if ((e = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal)) != cudaSuccess)
         return cuda_fail(e, "clbm_step: begin capture");

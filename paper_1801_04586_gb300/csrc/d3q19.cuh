@@ -84,14 +84,14 @@ __host__ __device__ constexpr uint32_t lowbias32(uint32_t x) {
 struct HalfSR { __half v; };
 struct BF16SR { __nv_bfloat16 v; };
 
-// Codec<T>: load a stored deviation as FP32; store an FP32 deviation. Formats
+// Codec<T>: load a stored deviation as FP32 (a plain load: see
+// grid_dependency_wait); store an FP32 deviation. Formats
 // with kStochastic round with a random dither r (from_f_sr), the others to
 // nearest even (from_f).
 template <typename T> struct Codec;
 template <> struct Codec<float> {
     static constexpr bool kStochastic = false;
-    static __device__ __forceinline__ float load(const float *p) { return __ldg(p); }
-    static __device__ __forceinline__ float load_plain(const float *p) { return *p; }
+    static __device__ __forceinline__ float load(const float *p) { return *p; }
     static __device__ __forceinline__ float from_f(float v) { return v; }
     static __device__ __forceinline__ float from_f_sr(float v, uint32_t) { return v; }
 };
@@ -112,8 +112,7 @@ __device__ __forceinline__ float2 unpack2_bf16(uint32_t w) {
 }
 template <> struct Codec<__half> {
     static constexpr bool kStochastic = false;
-    static __device__ __forceinline__ float load(const __half *p) { return __half2float(__ldg(p)); }
-    static __device__ __forceinline__ float load_plain(const __half *p) { return __half2float(*p); }
+    static __device__ __forceinline__ float load(const __half *p) { return __half2float(*p); }
     static __device__ __forceinline__ __half from_f(float v) { return __float2half_rn(v); }
     static __device__ __forceinline__ __half from_f_sr(float v, uint32_t) { return __float2half_rn(v); }
     static __device__ __forceinline__ uint32_t pair_rn(float hi, float lo) { return rn_pair_f16(hi, lo); }
@@ -121,8 +120,7 @@ template <> struct Codec<__half> {
 };
 template <> struct Codec<__nv_bfloat16> {
     static constexpr bool kStochastic = false;
-    static __device__ __forceinline__ float load(const __nv_bfloat16 *p) { return __bfloat162float(__ldg(p)); }
-    static __device__ __forceinline__ float load_plain(const __nv_bfloat16 *p) { return __bfloat162float(*p); }
+    static __device__ __forceinline__ float load(const __nv_bfloat16 *p) { return __bfloat162float(*p); }
     static __device__ __forceinline__ __nv_bfloat16 from_f(float v) { return __float2bfloat16_rn(v); }
     static __device__ __forceinline__ __nv_bfloat16 from_f_sr(float v, uint32_t) { return __float2bfloat16_rn(v); }
     static __device__ __forceinline__ uint32_t pair_rn(float hi, float lo) { return rn_pair_bf16(hi, lo); }
@@ -164,8 +162,7 @@ __device__ __forceinline__ uint32_t rn_pair_bf16(float hi, float lo) {
 // that node.
 template <> struct Codec<HalfSR> {
     static constexpr bool kStochastic = true;
-    static __device__ __forceinline__ float load(const HalfSR *p) { return __half2float(__ldg(&p->v)); }
-    static __device__ __forceinline__ float load_plain(const HalfSR *p) { return __half2float(p->v); }
+    static __device__ __forceinline__ float load(const HalfSR *p) { return __half2float(p->v); }
     static __device__ __forceinline__ HalfSR from_f(float v) { return HalfSR{__float2half_rn(v)}; }
     static __device__ __forceinline__ HalfSR from_f_sr(float v, uint32_t r, bool odd) {
         const uint32_t d = odd ? sr_pair_f16(v, 0.0f, r) >> 16 : sr_pair_f16(0.0f, v, r) & 0xffffu;
@@ -178,8 +175,7 @@ template <> struct Codec<HalfSR> {
 };
 template <> struct Codec<BF16SR> {
     static constexpr bool kStochastic = true;
-    static __device__ __forceinline__ float load(const BF16SR *p) { return __bfloat162float(__ldg(&p->v)); }
-    static __device__ __forceinline__ float load_plain(const BF16SR *p) { return __bfloat162float(p->v); }
+    static __device__ __forceinline__ float load(const BF16SR *p) { return __bfloat162float(p->v); }
     static __device__ __forceinline__ BF16SR from_f(float v) { return BF16SR{__float2bfloat16_rn(v)}; }
     static __device__ __forceinline__ BF16SR from_f_sr(float v, uint32_t r, bool odd) {
         const uint32_t d = odd ? sr_pair_bf16(v, 0.0f, r) >> 16 : sr_pair_bf16(0.0f, v, r) & 0xffffu;

@@ -12,8 +12,9 @@ namespace clbm {
 // warp-coalesced. At a row tail the second lane repeats the first node and is
 // not stored.
 template <typename S, int FM, bool WALLS>
-__global__ void __launch_bounds__(256) k_step2(const S *__restrict__ src, S *__restrict__ dst, Geom g, Rates r,
+__global__ void __launch_bounds__(256) k_step2(const S *src, S *__restrict__ dst, Geom g, Rates r,
                                                ForceArgs F, int *__restrict__ flag, uint32_t key) {
+    grid_dependency_wait();
     const int x0 = blockIdx.x * (2 * blockDim.x) + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z;
@@ -49,9 +50,11 @@ template <typename S, int FM>
 static cudaError_t step2_walls(const Launch &L, const void *src, void *dst, const Rates &r, const ForceArgs &F,
                                int *flag, uint32_t key) {
     if (L.g.walls)
-        k_step2<S, FM, true><<<L.grid, L.block, 0, L.stream>>>((const S *)src, (S *)dst, L.g, r, F, flag, key);
+        launch_overlapped(k_step2<S, FM, true>, L.grid, L.block, 0, L.stream, L.overlap, (const S *)src, (S *)dst,
+                          L.g, r, F, flag, key);
     else
-        k_step2<S, FM, false><<<L.grid, L.block, 0, L.stream>>>((const S *)src, (S *)dst, L.g, r, F, flag, key);
+        launch_overlapped(k_step2<S, FM, false>, L.grid, L.block, 0, L.stream, L.overlap, (const S *)src, (S *)dst,
+                          L.g, r, F, flag, key);
     return cudaGetLastError();
 }
 

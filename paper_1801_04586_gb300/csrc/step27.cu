@@ -61,7 +61,7 @@ __device__ __forceinline__ uint32_t state_load27(const S *src, const Geom &g, in
         for (int b = 0; b < 3; ++b)
 #pragma unroll
             for (int c = 0; c < 3; ++c)
-                h[a][b][c] = Codec<S>::load_plain(src + CLBM_IDX(g, (size_t)pop[a][b][c] * g.stride + off[a][b][c]));
+                h[a][b][c] = Codec<S>::load(src + CLBM_IDX(g, (size_t)pop[a][b][c] * g.stride + off[a][b][c]));
     return ((uint32_t)z * g.ny + y) * g.nx + x;
 }
 
@@ -81,8 +81,9 @@ __device__ __forceinline__ void scatter27(S *dst, const Geom &g, int x, int y, i
 }
 
 template <typename S, int FM, bool WALLS>
-__global__ void k_init27(S *dst, Geom g, int map, const float *__restrict__ rho, const float *__restrict__ u,
+__global__ void k_init27(S *dst, Geom g, int map, const float *rho, const float *u,
                          int64_t n, ForceArgs F) {
+    grid_dependency_wait();
     int x, y, z;
     if (!node27(g, x, y, z)) return;
     const uint32_t self = ((uint32_t)z * g.ny + y) * g.nx + x;
@@ -97,7 +98,8 @@ __global__ void k_init27(S *dst, Geom g, int map, const float *__restrict__ rho,
 }
 
 template <typename S, bool WALLS>
-__global__ void k_scatter27(S *dst, Geom g, int map, const float *__restrict__ f, int64_t n, int deviation) {
+__global__ void k_scatter27(S *dst, Geom g, int map, const float *f, int64_t n, int deviation) {
+    grid_dependency_wait();
     int x, y, z;
     if (!node27(g, x, y, z)) return;
     const uint32_t self = ((uint32_t)z * g.ny + y) * g.nx + x;
@@ -116,6 +118,7 @@ __global__ void k_scatter27(S *dst, Geom g, int map, const float *__restrict__ f
 
 template <typename S, bool WALLS>
 __global__ void k_gather27(const S *src, Geom g, int map, float *__restrict__ f, int64_t n, int deviation) {
+    grid_dependency_wait();
     int x, y, z;
     if (!node27(g, x, y, z)) return;
     float h[3][3][3];
@@ -133,6 +136,7 @@ __global__ void k_gather27(const S *src, Geom g, int map, float *__restrict__ f,
 template <typename S, int FM, bool WALLS>
 __global__ void k_macros27(const S *src, Geom g, int map, ForceArgs F, float *__restrict__ rho,
                            float *__restrict__ u, int64_t n) {
+    grid_dependency_wait();
     int x, y, z;
     if (!node27(g, x, y, z)) return;
     float h[3][3][3];
@@ -169,24 +173,30 @@ __global__ void k_moments27(const S *src, Geom g, int map, ForceArgs F, long lon
 cudaError_t launch_init27(int storage, const Launch &L, void *dst, const float *rho, const float *u, int64_t n,
                           const ForceArgs &F) {
     CLBM_Q27_STATE(storage, CLBM_Q27_FM(F.mode, {
-        if (L.g.walls) k_init27<S, FM, true><<<L.grid, L.block, 0, L.stream>>>((S *)dst, L.g, L.map, rho, u, n, F);
-        else k_init27<S, FM, false><<<L.grid, L.block, 0, L.stream>>>((S *)dst, L.g, L.map, rho, u, n, F);
+        if (L.g.walls) launch_overlapped(k_init27<S, FM, true>, L.grid, L.block, 0, L.stream, L.overlap, (S *)dst,
+                                         L.g, L.map, rho, u, n, F);
+        else launch_overlapped(k_init27<S, FM, false>, L.grid, L.block, 0, L.stream, L.overlap, (S *)dst, L.g, L.map,
+                               rho, u, n, F);
     }))
     return cudaGetLastError();
 }
 
 cudaError_t launch_scatter27(int storage, const Launch &L, void *dst, const float *f, int64_t n, int deviation) {
     CLBM_Q27_STATE(storage, {
-        if (L.g.walls) k_scatter27<S, true><<<L.grid, L.block, 0, L.stream>>>((S *)dst, L.g, L.map, f, n, deviation);
-        else k_scatter27<S, false><<<L.grid, L.block, 0, L.stream>>>((S *)dst, L.g, L.map, f, n, deviation);
+        if (L.g.walls) launch_overlapped(k_scatter27<S, true>, L.grid, L.block, 0, L.stream, L.overlap, (S *)dst,
+                                         L.g, L.map, f, n, deviation);
+        else launch_overlapped(k_scatter27<S, false>, L.grid, L.block, 0, L.stream, L.overlap, (S *)dst, L.g, L.map,
+                               f, n, deviation);
     })
     return cudaGetLastError();
 }
 
 cudaError_t launch_gather27(int storage, const Launch &L, const void *src, float *f, int64_t n, int deviation) {
     CLBM_Q27_STATE(storage, {
-        if (L.g.walls) k_gather27<S, true><<<L.grid, L.block, 0, L.stream>>>((const S *)src, L.g, L.map, f, n, deviation);
-        else k_gather27<S, false><<<L.grid, L.block, 0, L.stream>>>((const S *)src, L.g, L.map, f, n, deviation);
+        if (L.g.walls) launch_overlapped(k_gather27<S, true>, L.grid, L.block, 0, L.stream, L.overlap,
+                                         (const S *)src, L.g, L.map, f, n, deviation);
+        else launch_overlapped(k_gather27<S, false>, L.grid, L.block, 0, L.stream, L.overlap, (const S *)src, L.g,
+                               L.map, f, n, deviation);
     })
     return cudaGetLastError();
 }
@@ -194,8 +204,10 @@ cudaError_t launch_gather27(int storage, const Launch &L, const void *src, float
 cudaError_t launch_macros27(int storage, const Launch &L, const void *src, const ForceArgs &F, float *rho, float *u,
                             int64_t n) {
     CLBM_Q27_STATE(storage, CLBM_Q27_FM(F.mode, {
-        if (L.g.walls) k_macros27<S, FM, true><<<L.grid, L.block, 0, L.stream>>>((const S *)src, L.g, L.map, F, rho, u, n);
-        else k_macros27<S, FM, false><<<L.grid, L.block, 0, L.stream>>>((const S *)src, L.g, L.map, F, rho, u, n);
+        if (L.g.walls) launch_overlapped(k_macros27<S, FM, true>, L.grid, L.block, 0, L.stream, L.overlap,
+                                         (const S *)src, L.g, L.map, F, rho, u, n);
+        else launch_overlapped(k_macros27<S, FM, false>, L.grid, L.block, 0, L.stream, L.overlap, (const S *)src,
+                               L.g, L.map, F, rho, u, n);
     }))
     return cudaGetLastError();
 }

@@ -19,9 +19,9 @@ __device__ __forceinline__ void force27(const ForceArgs &F, const Geom &g, int z
     if (FM == kForceUniform) {
         fx = F.fx; fy = F.fy; fz = F.fz;
     } else if (FM == kForceProfileZ) {
-        fx = __ldg(F.profile + z); fy = __ldg(F.profile + g.nz + z); fz = __ldg(F.profile + 2 * g.nz + z);
+        fx = F.profile[z]; fy = F.profile[g.nz + z]; fz = F.profile[2 * g.nz + z];
     } else {
-        fx = __ldg(F.field + self); fy = __ldg(F.field + F.n + self); fz = __ldg(F.field + 2 * F.n + self);
+        fx = F.field[self]; fy = F.field[F.n + self]; fz = F.field[2 * F.n + self];
     }
     fx *= F.scale;
     fy *= F.scale;
@@ -60,8 +60,9 @@ __device__ __forceinline__ void flatten27(const float (&h)[3][3][3], float (&f)[
 }
 
 template <typename C, typename S, int FM, bool WALLS>
-__global__ void __launch_bounds__(256, 4) k_step27(const S *__restrict__ src, S *__restrict__ dst, Geom g, Rates27 r,
+__global__ void __launch_bounds__(256, 4) k_step27(const S *src, S *__restrict__ dst, Geom g, Rates27 r,
                                                 ForceArgs F, int *__restrict__ flag, uint32_t key) {
+    grid_dependency_wait();
     int x, y, z;
     if (!node27(g, x, y, z)) return;
     float h[3][3][3];
@@ -84,6 +85,7 @@ __global__ void __launch_bounds__(256, 4) k_step27(const S *__restrict__ src, S 
 template <typename C, typename S, int FM, bool WALLS, bool ODD>
 __global__ void __launch_bounds__(256) k_step27_aa(S *f, Geom g, Rates27 r, ForceArgs F, int *__restrict__ flag,
                                                    uint32_t key) {
+    grid_dependency_wait();
     int x, y, z;
     if (!node27(g, x, y, z)) return;
     const uint32_t self = ((uint32_t)z * g.ny + y) * g.nx + x;
@@ -173,9 +175,11 @@ cudaError_t launch_step27_with(int storage, const Launch &L, const void *src, vo
         if (staged)
             ;
         else if (L.g.walls)
-            k_step27<C, S, FM, true><<<L.grid, L.block, 0, L.stream>>>((const S *)src, (S *)dst, L.g, r, F, flag, key);
+            launch_overlapped(k_step27<C, S, FM, true>, L.grid, L.block, 0, L.stream, L.overlap, (const S *)src,
+                              (S *)dst, L.g, r, F, flag, key);
         else
-            k_step27<C, S, FM, false><<<L.grid, L.block, 0, L.stream>>>((const S *)src, (S *)dst, L.g, r, F, flag, key);
+            launch_overlapped(k_step27<C, S, FM, false>, L.grid, L.block, 0, L.stream, L.overlap, (const S *)src,
+                              (S *)dst, L.g, r, F, flag, key);
     }))
     return cudaGetLastError();
 }
@@ -185,11 +189,14 @@ cudaError_t launch_step27_aa_with(int storage, const Launch &L, void *f, const R
                                   int *flag, uint32_t key, bool odd) {
     CLBM_Q27_STORE(storage, CLBM_Q27_FM(F.mode, {
         if (!odd)
-            k_step27_aa<C, S, FM, false, false><<<L.grid, L.block, 0, L.stream>>>((S *)f, L.g, r, F, flag, key);
+            launch_overlapped(k_step27_aa<C, S, FM, false, false>, L.grid, L.block, 0, L.stream, L.overlap, (S *)f,
+                              L.g, r, F, flag, key);
         else if (L.g.walls)
-            k_step27_aa<C, S, FM, true, true><<<L.grid, L.block, 0, L.stream>>>((S *)f, L.g, r, F, flag, key);
+            launch_overlapped(k_step27_aa<C, S, FM, true, true>, L.grid, L.block, 0, L.stream, L.overlap, (S *)f,
+                              L.g, r, F, flag, key);
         else
-            k_step27_aa<C, S, FM, false, true><<<L.grid, L.block, 0, L.stream>>>((S *)f, L.g, r, F, flag, key);
+            launch_overlapped(k_step27_aa<C, S, FM, false, true>, L.grid, L.block, 0, L.stream, L.overlap, (S *)f,
+                              L.g, r, F, flag, key);
     }))
     return cudaGetLastError();
 }

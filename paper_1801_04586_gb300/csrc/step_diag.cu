@@ -46,9 +46,9 @@ __device__ __forceinline__ void force_diag(const ForceArgs &F, const Geom &g, in
     if (FM == kForceUniform) {
         fx = F.fx; fy = F.fy; fz = F.fz;
     } else if (FM == kForceProfileZ) {
-        fx = __ldg(F.profile + z); fy = __ldg(F.profile + g.nz + z); fz = __ldg(F.profile + 2 * g.nz + z);
+        fx = F.profile[z]; fy = F.profile[g.nz + z]; fz = F.profile[2 * g.nz + z];
     } else {
-        fx = __ldg(F.field + self); fy = __ldg(F.field + F.n + self); fz = __ldg(F.field + 2 * F.n + self);
+        fx = F.field[self]; fy = F.field[F.n + self]; fz = F.field[2 * F.n + self];
     }
     fx *= F.scale;
     fy *= F.scale;
@@ -60,11 +60,12 @@ __device__ __forceinline__ void force_diag(const ForceArgs &F, const Geom &g, in
 constexpr int kDiagZ = 4;
 
 template <typename S, int FM, bool WALLS>
-__global__ void __launch_bounds__(512, 2) k_step_diag(const S *__restrict__ src, S *__restrict__ dst, Geom g,
+__global__ void __launch_bounds__(512, 2) k_step_diag(const S *src, S *__restrict__ dst, Geom g,
                                                       Rates r, ForceArgs F, int *__restrict__ flag,
                                                       unsigned long long *__restrict__ acc,
                                                       unsigned long long *__restrict__ acc_prev, double *out_prev,
                                                       double add0, uint32_t key, int zb, int ze) {
+    grid_dependency_wait();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z0 = zb + blockIdx.z * kDiagZ;
@@ -120,10 +121,12 @@ static cudaError_t diag_walls(const Launch &L, const void *src, void *dst, const
     if (L.zs != 1 || zb < 0 || np < 1 || zb + np > L.g.nz) return cudaErrorInvalidValue;
     const dim3 grid(L.grid.x, L.grid.y, (np + kDiagZ - 1) / kDiagZ);
     if (L.g.walls)
-        k_step_diag<S, FM, true><<<grid, L.block, 0, L.stream>>>((const S *)src, (S *)dst, L.g, r, F, flag, d.acc,
+        launch_overlapped(k_step_diag<S, FM, true>, grid, L.block, 0, L.stream, L.overlap, (const S *)src, (S *)dst,
+                          L.g, r, F, flag, d.acc,
                                                                  d.acc_prev, d.out_prev, d.add0, key, zb, zb + np);
     else
-        k_step_diag<S, FM, false><<<grid, L.block, 0, L.stream>>>((const S *)src, (S *)dst, L.g, r, F, flag, d.acc,
+        launch_overlapped(k_step_diag<S, FM, false>, grid, L.block, 0, L.stream, L.overlap, (const S *)src, (S *)dst,
+                          L.g, r, F, flag, d.acc,
                                                                   d.acc_prev, d.out_prev, d.add0, key, zb, zb + np);
     return cudaGetLastError();
 }

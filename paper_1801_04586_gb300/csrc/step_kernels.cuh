@@ -28,13 +28,13 @@ __device__ __forceinline__ void force_at(const ForceArgs &F, const Geom &g, int 
     if (FM == kForceUniform) {
         fx = F.fx; fy = F.fy; fz = F.fz;
     } else if (FM == kForceProfileZ) {
-        fx = __ldg(F.profile + z);
-        fy = __ldg(F.profile + g.nz + z);
-        fz = __ldg(F.profile + 2 * g.nz + z);
+        fx = F.profile[z];
+        fy = F.profile[g.nz + z];
+        fz = F.profile[2 * g.nz + z];
     } else {
-        fx = __ldg(F.field + self);
-        fy = __ldg(F.field + F.n + self);
-        fz = __ldg(F.field + 2 * F.n + self);
+        fx = F.field[self];
+        fy = F.field[F.n + self];
+        fz = F.field[2 * F.n + self];
     }
     fx *= F.scale;
     fy *= F.scale;
@@ -48,8 +48,9 @@ __device__ __forceinline__ void force_at(const ForceArgs &F, const Geom &g, int 
 namespace clbm {
 
 template <typename C, typename S, int FM, bool WALLS>
-__global__ void __launch_bounds__(512) k_step(const S *__restrict__ src, S *__restrict__ dst, Geom g, Rates r,
+__global__ void __launch_bounds__(512) k_step(const S *src, S *__restrict__ dst, Geom g, Rates r,
                                               ForceArgs F, int *__restrict__ flag, uint32_t key) {
+    grid_dependency_wait();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z;
@@ -84,6 +85,7 @@ __global__ void __launch_bounds__(512) k_step(const S *__restrict__ src, S *__re
 template <typename C, typename S, int FM, bool WALLS, bool ODD>
 __global__ void __launch_bounds__(512, sizeof(S) == 2 ? 2 : 0) k_step_aa(S *f, Geom g, Rates r, ForceArgs F, int *__restrict__ flag,
                                                  uint32_t key) {
+    grid_dependency_wait();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z;
@@ -127,9 +129,11 @@ static cudaError_t step_walls_t(const Launch &L, const void *src, void *dst, con
         if (L.staged && launch_step_tma<19, C, S, FM>(L, src, dst, r, F, flag, key, e)) return e;
     }
     if (L.g.walls)
-        k_step<C, S, FM, true><<<L.grid, L.block, 0, L.stream>>>((const S *)src, (S *)dst, L.g, r, F, flag, key);
+        launch_overlapped(k_step<C, S, FM, true>, L.grid, L.block, 0, L.stream, L.overlap, (const S *)src, (S *)dst,
+                          L.g, r, F, flag, key);
     else
-        k_step<C, S, FM, false><<<L.grid, L.block, 0, L.stream>>>((const S *)src, (S *)dst, L.g, r, F, flag, key);
+        launch_overlapped(k_step<C, S, FM, false>, L.grid, L.block, 0, L.stream, L.overlap, (const S *)src, (S *)dst,
+                          L.g, r, F, flag, key);
     return cudaGetLastError();
 }
 
@@ -160,11 +164,14 @@ template <typename C, typename S, int FM>
 static cudaError_t step_aa_walls_t(const Launch &L, void *f, const Rates &r, const ForceArgs &F, int *flag,
                                    uint32_t key, bool odd) {
     if (!odd)
-        k_step_aa<C, S, FM, false, false><<<L.grid, L.block, 0, L.stream>>>((S *)f, L.g, r, F, flag, key);
+        launch_overlapped(k_step_aa<C, S, FM, false, false>, L.grid, L.block, 0, L.stream, L.overlap, (S *)f, L.g, r,
+                          F, flag, key);
     else if (L.g.walls)
-        k_step_aa<C, S, FM, true, true><<<L.grid, L.block, 0, L.stream>>>((S *)f, L.g, r, F, flag, key);
+        launch_overlapped(k_step_aa<C, S, FM, true, true>, L.grid, L.block, 0, L.stream, L.overlap, (S *)f, L.g, r,
+                          F, flag, key);
     else
-        k_step_aa<C, S, FM, false, true><<<L.grid, L.block, 0, L.stream>>>((S *)f, L.g, r, F, flag, key);
+        launch_overlapped(k_step_aa<C, S, FM, false, true>, L.grid, L.block, 0, L.stream, L.overlap, (S *)f, L.g, r,
+                          F, flag, key);
     return cudaGetLastError();
 }
 

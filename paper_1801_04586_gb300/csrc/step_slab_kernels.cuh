@@ -19,8 +19,9 @@ namespace clbm {
 // (node0 + local index), so a slab stores exactly what the undivided lattice
 // stores.
 template <typename C, typename S, int FM, bool WALLS>
-__global__ void __launch_bounds__(512) k_step_slab(const S *__restrict__ src, S *__restrict__ dst, Geom g, Rates r,
+__global__ void __launch_bounds__(512) k_step_slab(const S *src, S *__restrict__ dst, Geom g, Rates r,
                                                    ForceArgs F, int *__restrict__ flag, uint32_t key, int z0, int zs) {
+    grid_dependency_wait();
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = z0 + (int)blockIdx.z * zs;
@@ -58,10 +59,12 @@ static cudaError_t step_slab_walls_t(const Launch &L, const void *src, void *dst
     dim3 grid = L.grid;
     grid.z = (unsigned)nplanes;
     if (L.g.walls)
-        k_step_slab<C, S, FM, true><<<grid, L.block, 0, L.stream>>>((const S *)src, (S *)dst, L.g, r, F, flag, key,
+        launch_overlapped(k_step_slab<C, S, FM, true>, grid, L.block, 0, L.stream, L.overlap, (const S *)src,
+                          (S *)dst, L.g, r, F, flag, key,
                                                                     z0, zs);
     else
-        k_step_slab<C, S, FM, false><<<grid, L.block, 0, L.stream>>>((const S *)src, (S *)dst, L.g, r, F, flag, key,
+        launch_overlapped(k_step_slab<C, S, FM, false>, grid, L.block, 0, L.stream, L.overlap, (const S *)src,
+                          (S *)dst, L.g, r, F, flag, key,
                                                                      z0, zs);
     return cudaGetLastError();
 }
