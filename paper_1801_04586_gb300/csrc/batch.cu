@@ -277,8 +277,8 @@ Launch domain_launch(const clbm_batch *b, int d) {
     const Geom &g = b->descs[d].g;
     Launch L;
     L.g = g;
-    const int bx = g.nx >= 128 ? 128 : ((g.nx + 31) / 32) * 32;
-    const int by = std::max(1, std::min(g.ny, 256 / bx));
+    const int bx = default_block_x(g.nx);
+    const int by = std::max(1, std::min(g.ny, 128 / bx));
     L.block = dim3(bx, by, 1);
     L.grid = dim3((g.nx + bx - 1) / bx, (g.ny + by - 1) / by, g.nz);
     L.stream = b->stream;

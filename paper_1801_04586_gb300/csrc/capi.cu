@@ -321,8 +321,8 @@ int clbm_create(const clbm_params *p, void *stream, clbm_ctx **out) {
     if (p->model != CLBM_MODEL_CASCADED && p->variant == 2)
         return fail(CLBM_ERR_ARG, "clbm_create: the SRT and MRT models run one node per thread");
     int bx = p->block_x, by = p->block_y;
-    if (bx == 0) bx = p->nx >= 128 ? 128 : ((p->nx + 31) / 32) * 32;
-    if (by == 0) by = std::max(1, std::min(p->ny, 256 / bx));
+    if (bx == 0) bx = default_block_x(p->nx);
+    if (by == 0) by = std::max(1, std::min(p->ny, 128 / bx));
     if (bx < 32 || bx % 32 != 0 || by < 1 || bx * by > 512)
         return fail(CLBM_ERR_ARG, "clbm_create: block_x must be a multiple of 32 and block_x*block_y <= 512");
     if ((p->ny + by - 1) / by > 65535) return fail(CLBM_ERR_ARG, "clbm_create: ny / block_y exceeds grid limit");

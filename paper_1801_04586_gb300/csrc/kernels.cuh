@@ -54,6 +54,26 @@ struct ForceArgs {
     float scale;             // time factor e^{-gamma t} of the step (1 for a static force)
 };
 
+// Default block of the one-node kernels: about 128 threads, of the width
+// (a multiple of 32, at most 224) that leaves the fewest idle lanes in a row
+// of nx nodes; 128 among equals, else the widest. Against a fixed 128 x 2
+// (us a step, FP32): 150 x 91 x 61 with y walls and a force field 25.4 -> 22.5
+// (160 x 1; half of 256 lanes were idle), 200 x 180 x 160 with z walls 149 ->
+// 139 (224 x 1), D3Q27 at 192 x 176 x 160 192 -> 181 (192 x 1), 256^3 380.6 ->
+// 376 (128 x 1: smaller blocks leave less idle while the last one finishes).
+inline int default_block_x(int nx) {
+    int best = 32;
+    int64_t pad = INT64_MAX;
+    for (int bx = 32; bx <= 224; bx += 32) {
+        const int64_t w = ((int64_t)nx + bx - 1) / bx * bx;
+        if (w < pad || (w == pad && best != 128)) {
+            pad = w;
+            best = bx;
+        }
+    }
+    return best;
+}
+
 struct Launch {
     Geom g;
     dim3 block, grid;  // grid of the one-node-per-thread kernels
