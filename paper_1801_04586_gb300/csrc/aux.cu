@@ -67,7 +67,7 @@ __device__ __forceinline__ uint32_t pull_node(const S *src, const Geom &g, int x
     int pop[kQ];
     state_slots<WALLS>(g, x, y, z, map, off, pop);
 #pragma unroll
-    for (int i = 0; i < kQ; ++i) h[i] = Codec<S>::load(src + CLBM_IDX(g, (size_t)pop[i] * g.stride + off[i]));
+    for (int i = 0; i < kQ; ++i) h[i] = Codec<S>::load_plain(src + CLBM_IDX(g, (size_t)pop[i] * g.stride + off[i]));
     return ((uint32_t)z * g.ny + y) * g.nx + x;
 }
 

@@ -114,8 +114,10 @@ __global__ void __launch_bounds__(512) k_batch_step(const S *A, S *__restrict__ 
 // population i to (i, x + e_i), or (ibar, x) across a wall. The same tiles,
 // domain table and collision as k_batch_step, so the batch stores the bits of
 // the A/B batch and of each domain stepped alone.
+// The even kind with FP32 wants 84 registers: capped at two blocks of 512 (64)
+// an in-place step of the benchmark's 64 domains takes 1005 instead of 1088 us.
 template <typename S, bool SMEM, bool ODD>
-__global__ void __launch_bounds__(512) k_batch_step_aa(S *A, const DomainDesc *__restrict__ doms, int ndom,
+__global__ void __launch_bounds__(512, ODD || sizeof(S) == 2 ? 0 : 2) k_batch_step_aa(S *A, const DomainDesc *__restrict__ doms, int ndom,
                                                        const int4 *__restrict__ tiles, int ntiles,
                                                        int *__restrict__ flag) {
     extern __shared__ DomainDesc sdom[];

@@ -84,14 +84,34 @@ __host__ __device__ constexpr uint32_t lowbias32(uint32_t x) {
 struct HalfSR { __half v; };
 struct BF16SR { __nv_bfloat16 v; };
 
-// Codec<T>: load a stored deviation as FP32 (a plain load: see
-// grid_dependency_wait); store an FP32 deviation. Formats
+// A load from global memory that the compiler may move across other accesses
+// (each value is read once, before the store that depends on it), but not
+// before grid_dependency_wait, as it could a load through the read-only path.
+__device__ __forceinline__ float ld_state(const float *p) {
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ __half ld_state(const __half *p) {
+    __half_raw v;
+    asm volatile("ld.global.u16 %0, [%1];" : "=h"(v.x) : "l"(p));
+    return __half(v);
+}
+__device__ __forceinline__ __nv_bfloat16 ld_state(const __nv_bfloat16 *p) {
+    __nv_bfloat16_raw v;
+    asm volatile("ld.global.u16 %0, [%1];" : "=h"(v.x) : "l"(p));
+    return __nv_bfloat16(v);
+}
+
+// Codec<T>: load a stored deviation as FP32 (load: global memory, ld_state;
+// load_plain: any memory); store an FP32 deviation. Formats
 // with kStochastic round with a random dither r (from_f_sr), the others to
 // nearest even (from_f).
 template <typename T> struct Codec;
 template <> struct Codec<float> {
     static constexpr bool kStochastic = false;
-    static __device__ __forceinline__ float load(const float *p) { return *p; }
+    static __device__ __forceinline__ float load(const float *p) { return ld_state(p); }
+    static __device__ __forceinline__ float load_plain(const float *p) { return *p; }
     static __device__ __forceinline__ float from_f(float v) { return v; }
     static __device__ __forceinline__ float from_f_sr(float v, uint32_t) { return v; }
 };
@@ -112,7 +132,8 @@ __device__ __forceinline__ float2 unpack2_bf16(uint32_t w) {
 }
 template <> struct Codec<__half> {
     static constexpr bool kStochastic = false;
-    static __device__ __forceinline__ float load(const __half *p) { return __half2float(*p); }
+    static __device__ __forceinline__ float load(const __half *p) { return __half2float(ld_state(p)); }
+    static __device__ __forceinline__ float load_plain(const __half *p) { return __half2float(*p); }
     static __device__ __forceinline__ __half from_f(float v) { return __float2half_rn(v); }
     static __device__ __forceinline__ __half from_f_sr(float v, uint32_t) { return __float2half_rn(v); }
     static __device__ __forceinline__ uint32_t pair_rn(float hi, float lo) { return rn_pair_f16(hi, lo); }
@@ -120,7 +141,8 @@ template <> struct Codec<__half> {
 };
 template <> struct Codec<__nv_bfloat16> {
     static constexpr bool kStochastic = false;
-    static __device__ __forceinline__ float load(const __nv_bfloat16 *p) { return __bfloat162float(*p); }
+    static __device__ __forceinline__ float load(const __nv_bfloat16 *p) { return __bfloat162float(ld_state(p)); }
+    static __device__ __forceinline__ float load_plain(const __nv_bfloat16 *p) { return __bfloat162float(*p); }
     static __device__ __forceinline__ __nv_bfloat16 from_f(float v) { return __float2bfloat16_rn(v); }
     static __device__ __forceinline__ __nv_bfloat16 from_f_sr(float v, uint32_t) { return __float2bfloat16_rn(v); }
     static __device__ __forceinline__ uint32_t pair_rn(float hi, float lo) { return rn_pair_bf16(hi, lo); }
@@ -162,7 +184,8 @@ __device__ __forceinline__ uint32_t rn_pair_bf16(float hi, float lo) {
 // that node.
 template <> struct Codec<HalfSR> {
     static constexpr bool kStochastic = true;
-    static __device__ __forceinline__ float load(const HalfSR *p) { return __half2float(p->v); }
+    static __device__ __forceinline__ float load(const HalfSR *p) { return __half2float(ld_state(&p->v)); }
+    static __device__ __forceinline__ float load_plain(const HalfSR *p) { return __half2float(p->v); }
     static __device__ __forceinline__ HalfSR from_f(float v) { return HalfSR{__float2half_rn(v)}; }
     static __device__ __forceinline__ HalfSR from_f_sr(float v, uint32_t r, bool odd) {
         const uint32_t d = odd ? sr_pair_f16(v, 0.0f, r) >> 16 : sr_pair_f16(0.0f, v, r) & 0xffffu;
@@ -175,7 +198,8 @@ template <> struct Codec<HalfSR> {
 };
 template <> struct Codec<BF16SR> {
     static constexpr bool kStochastic = true;
-    static __device__ __forceinline__ float load(const BF16SR *p) { return __bfloat162float(p->v); }
+    static __device__ __forceinline__ float load(const BF16SR *p) { return __bfloat162float(ld_state(&p->v)); }
+    static __device__ __forceinline__ float load_plain(const BF16SR *p) { return __bfloat162float(p->v); }
     static __device__ __forceinline__ BF16SR from_f(float v) { return BF16SR{__float2bfloat16_rn(v)}; }
     static __device__ __forceinline__ BF16SR from_f_sr(float v, uint32_t r, bool odd) {
         const uint32_t d = odd ? sr_pair_bf16(v, 0.0f, r) >> 16 : sr_pair_bf16(0.0f, v, r) & 0xffffu;
@@ -462,15 +486,32 @@ __device__ __forceinline__ float recip_nr(float x) {
 __device__ __forceinline__ f2 recip_nr(f2 x) { return mk2(recip_nr(x.v.x), recip_nr(x.v.y)); }
 __device__ __forceinline__ f1 recip_nr(f1 x) { return f1{recip_nr(x.v)}; }
 
+// Correctly rounded 1/x of both lanes: recip_nr's result r is within an ulp, so
+// one more residual step r + r (1 - x r), its residual exact in the fused
+// multiply-add, rounds to the nearest (Markstein 1990, IBM J. Res. Dev. 34);
+// verified against the division for every density in (0.1, 1.9). Lanes outside
+// the normal range of densities (a state the instability flag reports) divide.
+__device__ __forceinline__ f2 recip_exact(f2 x) {
+    f2 r = recip_nr(x);
+    const f2 e = fmaf(-x, r, mk2(1.0f));
+    r = fmaf(r, e, r);
+    const bool odd0 = !(x.v.x > 0.0625f && x.v.x < 16.0f), odd1 = !(x.v.y > 0.0625f && x.v.y < 16.0f);
+    if (odd0) r.v.x = 1.0f / x.v.x;
+    if (odd1) r.v.y = 1.0f / x.v.y;
+    return r;
+}
+
 // The collision's 1/rho: recip_nr when FR (16-bit storage, whose steps are
-// bound by instruction issue: 3 to 6 % faster), the IEEE division otherwise
-// (FP32 steps are bound by DRAM; there the shorter sequence let the compiler
-// stretch live ranges, 58 -> 81 registers in the in-place odd step, and
-// measured 1-4 % slower).
+// bound by instruction issue: 3 to 6 % faster), the correctly rounded quotient
+// otherwise, for a pair of nodes without the division's instruction sequence.
 template <bool FR, typename T>
 __device__ __forceinline__ T recip_of(T x) {
     if constexpr (FR)
         return recip_nr(x);
+    else if constexpr (std::is_same<T, f2>::value)
+        return recip_exact(x);
+    else if constexpr (std::is_same<T, f1>::value)
+        return f1{1.0f / x.v};
     else
         return 1.0f / x;
 }
@@ -593,16 +634,33 @@ __device__ __forceinline__ T collide_t(T (&h)[kQ], T Fx, T Fy, T Fz, const Rates
     } else if constexpr (std::is_same<T, f1>::value) {
         if (j_out) *j_out = make_float3(jx.v, jy.v, jz.v);
     }
-    EqDevT<T> e;
-    eq_dev(drho, rho, jx, jy, jz, ux, uy, uz, e);
-
     // non-equilibrium raw moments R = dT - (rho G - M w); R000 = 0, R100 = -Fx/2, ...
     const T hFx = 0.5f * Fx, hFy = 0.5f * Fy, hFz = 0.5f * Fz;
-    T r110 = k.m110 - e.d110, r101 = k.m101 - e.d101, r011 = k.m011 - e.d011;
-    T r200 = k.m200 - e.d200, r020 = k.m020 - e.d020, r002 = k.m002 - e.d002;
-    T r120 = k.m120 - e.d120, r102 = k.m102 - e.d102, r210 = k.m210 - e.d210;
-    T r201 = k.m201 - e.d201, r012 = k.m012 - e.d012, r021 = k.m021 - e.d021;
-    T r220 = k.m220 - e.d220, r202 = k.m202 - e.d202, r022 = k.m022 - e.d022;
+    EqDevT<T> e;        // FR: all 15 equilibrium deviations, subtracted here and added back at the end
+    T Xc, Yc, Zc;       // !FR: factors u^2 + c_s^2 of the products that are fused into the sums instead
+    T r110, r101, r011, r200, r020, r002, r120, r102, r210, r201, r012, r021, r220, r202, r022;
+    if constexpr (FR) {
+        eq_dev(drho, rho, jx, jy, jz, ux, uy, uz, e);
+        r110 = k.m110 - e.d110; r101 = k.m101 - e.d101; r011 = k.m011 - e.d011;
+        r120 = k.m120 - e.d120; r102 = k.m102 - e.d102; r210 = k.m210 - e.d210;
+        r201 = k.m201 - e.d201; r012 = k.m012 - e.d012; r021 = k.m021 - e.d021;
+    } else {
+        const T X = ux * ux, Y = uy * uy, Z = uz * uz;
+        Xc = X + kC; Yc = Y + kC; Zc = Z + kC;
+        const T njx = -jx, njy = -jy, njz = -jz;
+        r110 = fmaf(njx, uy, k.m110); r101 = fmaf(njx, uz, k.m101); r011 = fmaf(njy, uz, k.m011);
+        r120 = fmaf(njx, Yc, k.m120); r102 = fmaf(njx, Zc, k.m102); r210 = fmaf(njy, Xc, k.m210);
+        r201 = fmaf(njz, Xc, k.m201); r012 = fmaf(njy, Zc, k.m012); r021 = fmaf(njz, Yc, k.m021);
+        const T dc = drho * kC, dc2 = drho * kC2;
+        e.d200 = fmaf(jx, ux, dc); e.d020 = fmaf(jy, uy, dc); e.d002 = fmaf(jz, uz, dc);
+        // X Y + c (X + Y) = X (Y + c) + c Y
+        const T cY = kC * Y, cZ = kC * Z;
+        e.d220 = fmaf(rho, fmaf(X, Yc, cY), dc2);
+        e.d202 = fmaf(rho, fmaf(X, Zc, cZ), dc2);
+        e.d022 = fmaf(rho, fmaf(Y, Zc, cZ), dc2);
+    }
+    r200 = k.m200 - e.d200; r020 = k.m020 - e.d020; r002 = k.m002 - e.d002;
+    r220 = k.m220 - e.d220; r202 = k.m202 - e.d202; r022 = k.m022 - e.d022;
 
     // D = N(u) R: x shift on (000,100,200) (010,110,210) (001,101,201) (020,120,220) (002,102,202)
     r200 = fmaf(ux, Fx, r200);                 // R000 = 0, R100 = -Fx/2
@@ -661,22 +719,27 @@ __device__ __forceinline__ T collide_t(T (&h)[kQ], T Fx, T Fy, T Fz, const Rates
     MomentsT<T> q;
     q.m000 = drho;
     q.m100 = jx + hFx; q.m010 = jy + hFy; q.m001 = jz + hFz;
-    q.m110 = r110 + e.d110; q.m101 = r101 + e.d101; q.m011 = r011 + e.d011;
+    if constexpr (FR) {
+        q.m110 = r110 + e.d110; q.m101 = r101 + e.d101; q.m011 = r011 + e.d011;
+        q.m120 = r120 + e.d120; q.m102 = r102 + e.d102; q.m210 = r210 + e.d210;
+        q.m201 = r201 + e.d201; q.m012 = r012 + e.d012; q.m021 = r021 + e.d021;
+    } else {
+        q.m110 = fmaf(jx, uy, r110); q.m101 = fmaf(jx, uz, r101); q.m011 = fmaf(jy, uz, r011);
+        q.m120 = fmaf(jx, Yc, r120); q.m102 = fmaf(jx, Zc, r102); q.m210 = fmaf(jy, Xc, r210);
+        q.m201 = fmaf(jz, Xc, r201); q.m012 = fmaf(jy, Zc, r012); q.m021 = fmaf(jz, Yc, r021);
+    }
     q.m200 = r200 + e.d200; q.m020 = r020 + e.d020; q.m002 = r002 + e.d002;
-    q.m120 = r120 + e.d120; q.m102 = r102 + e.d102; q.m210 = r210 + e.d210;
-    q.m201 = r201 + e.d201; q.m012 = r012 + e.d012; q.m021 = r021 + e.d021;
     q.m220 = r220 + e.d220; q.m202 = r202 + e.d202; q.m022 = r022 + e.d022;
     inverse_moments(q, h);
     return drho;
 }
 
-// The collision of one node (float) or two (f2). With FR (16-bit storage) a
-// float node runs on f1, rounding every operation on its own, so that it
-// matches the f2 form bit for bit; FP32 storage keeps the compiler's fused
-// multiply-adds.
+// The collision of one node (float) or two (f2). A float node runs on f1,
+// rounding every operation on its own, so that it matches the f2 form bit for
+// bit, whichever kernel steps it.
 template <bool FR = false, typename T>
 __device__ __forceinline__ T collide(T (&h)[kQ], T Fx, T Fy, T Fz, const Rates &r, float3 *j_out = nullptr) {
-    if constexpr (FR && std::is_same<T, float>::value) {
+    if constexpr (std::is_same<T, float>::value) {
         f1 g[kQ];
 #pragma unroll
         for (int i = 0; i < kQ; ++i) g[i].v = h[i];

@@ -347,7 +347,7 @@ __device__ __forceinline__ void compute_tile(const S *src, S *__restrict__ dst, 
 #pragma unroll
             for (int i = 0; i < kQ; ++i) {
                 const uint32_t j = ex19(i) > 0 ? sm : (ex19(i) < 0 ? sp : n);
-                h[i] = Codec<S>::load(stage + i * TN + CLBM_SIDX(g, j, tile));
+                h[i] = Codec<S>::load_plain(stage + i * TN + CLBM_SIDX(g, j, tile));
             }
             if (WALLS && any) {
                 const bool bb[kQ] = {false,
@@ -371,7 +371,7 @@ __device__ __forceinline__ void compute_tile(const S *src, S *__restrict__ dst, 
 #pragma unroll
                     for (int c = 0; c < 3; ++c) {
                         const uint32_t j = a == 1 ? sm : (a == 2 ? sp : n);
-                        h[a][b][c] = Codec<S>::load(stage + q27_index(a, b, c) * TN + CLBM_SIDX(g, j, tile));
+                        h[a][b][c] = Codec<S>::load_plain(stage + q27_index(a, b, c) * TN + CLBM_SIDX(g, j, tile));
                     }
             if (WALLS && any) {
                 const bool bx[3] = {false, xl, xh}, by[3] = {false, yl, yh}, bz[3] = {false, zl, zh};
@@ -502,11 +502,11 @@ __device__ __forceinline__ void compute_tile_pairs(const S *src, S *dst, const G
                     Codec<S>::unpack2(*reinterpret_cast<const uint32_t *>(row + CLBM_SIDX(g, n, tile - 1u)));
                 h[i] = f2{v};
             } else if (ex19(i) > 0) {  // from x - 1
-                h[i] = mk2(Codec<S>::load(row + CLBM_SIDX(g, sm0, tile)),
-                           Codec<S>::load(row + CLBM_SIDX(g, n, tile)));
+                h[i] = mk2(Codec<S>::load_plain(row + CLBM_SIDX(g, sm0, tile)),
+                           Codec<S>::load_plain(row + CLBM_SIDX(g, n, tile)));
             } else {                   // from x + 1
-                h[i] = mk2(Codec<S>::load(row + CLBM_SIDX(g, n + 1u, tile)),
-                           Codec<S>::load(row + CLBM_SIDX(g, sp1, tile)));
+                h[i] = mk2(Codec<S>::load_plain(row + CLBM_SIDX(g, n + 1u, tile)),
+                           Codec<S>::load_plain(row + CLBM_SIDX(g, sp1, tile)));
             }
         }
         if (WALLS && MODE != kTileAAEven) {  // (the in-place even step reads only its own slots)
