@@ -112,7 +112,9 @@ extern "C" {
  *      and the cascaded D3Q19 in-place (AA) steps with 16-bit storage, stage
  *      the rows they read in shared memory with bulk asynchronous copies
  *      where the geometry allows (nx <= 1024, nx a multiple of 8; D3Q27 not
- *      with a force field), one node per thread otherwise; 1: always one node per thread,
+ *      with a force field); cascaded D3Q19 A/B steps with FP32 storage on
+ *      lattices of 100,000 nodes or more collide two adjacent nodes per thread
+ *      (unless block_x or block_y is given); one node per thread otherwise; 1: always one node per thread,
  *      plain loads (block_x, block_y apply); 2: two nodes per thread (x and
  *      x + block_x), collided together with the FP32x2 instructions (D3Q19
  *      only; measured slower on GB300 for every storage format, kept as an
@@ -184,7 +186,7 @@ typedef struct clbm_info {
     int32_t storage;
     int32_t block_x, block_y; /* block shape in use */
     double s2;                /* 1/(3 nu + 1/2) */
-    int32_t nodes_per_thread; /* of the step kernel: 1 or 2 */
+    int32_t nodes_per_thread; /* 2 with variant 2, else 1 (also where variant 0 collides adjacent nodes in pairs) */
     int32_t q;                /* 19 or 27 */
     int32_t pattern;          /* CLBM_PATTERN_AB or CLBM_PATTERN_AA */
     int32_t buffers;          /* population buffers held: 2 (A/B) or 1 (AA) */

@@ -86,6 +86,7 @@ struct clbm_ctx {
     int64_t steps_done;
     double gamma;         // force decay rate (clbm_set_force_decay)
     bool packed;          // step kernel with two nodes per thread (FP32x2 arithmetic)
+    bool pairs;           // FP32 steps with two adjacent nodes per thread (step_pair.cu)
     bool staged;          // steps with rows staged in shared memory by bulk copies (variant 0; see clbm_create)
     int q;                // 19 (Appendix A) or 27 (Sec. II)
     bool aa;              // in-place (AA) pattern: one population buffer, step kind by parity
@@ -153,6 +154,7 @@ Launch launch_of(const clbm_ctx *c) {
     L.stream = c->stream;
     L.packed = false;
     L.staged = c->staged;
+    L.pairs = c->pairs;
     // A/B: the pull map (through the halo planes for a z-slab); AA: natural
     // slots after an even number of steps, the odd step's swapped pull map
     // after an odd number.
@@ -357,6 +359,9 @@ int clbm_create(const clbm_params *p, void *stream, clbm_ctx **out) {
     // staged: A/B steps, and the cascaded D3Q19 in-place step (node pairs)
     c->staged = p->variant == 0 &&
                 (p->pattern != CLBM_PATTERN_AA || (q == 19 && p->model == CLBM_MODEL_CASCADED));
+    // pairs: FP32 A/B cascaded D3Q19 steps, unless the caller chose a block shape of the one-node kernel
+    c->pairs = q == 19 && p->variant == 0 && p->storage == CLBM_STORAGE_F32 && p->pattern == CLBM_PATTERN_AB &&
+               p->model == CLBM_MODEL_CASCADED && !p->slab && p->block_x == 0 && p->block_y == 0 && step_pairs(c->g);
     c->aa = p->pattern == CLBM_PATTERN_AA;
     c->model = p->model;
     c->rates27.om2 = c->rates.om2;

@@ -70,6 +70,7 @@ static cudaError_t step2_force(const Launch &L, const void *src, void *dst, cons
 
 cudaError_t launch_step(int storage, const Launch &L, const void *src, void *dst, const Rates &r,
                         const ForceArgs &F, int *flag, uint32_t key) {
+    if (L.pairs && storage == 0) return launch_step_pair(L, src, dst, r, F, flag);
     if (!L.packed) return launch_step_with<Cascaded>(storage, L, src, dst, r, F, flag, key);
     switch (storage) {
         case 0: return step2_force<float>(L, src, dst, r, F, flag, key);

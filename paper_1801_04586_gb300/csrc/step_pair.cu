@@ -1,0 +1,45 @@
+// step_pair.cu -- launch of the FP32 node-pair step (step_pair.cuh).
+#include "step_pair.cuh"
+
+namespace clbm {
+
+// From 100,000 nodes on: two to three warps of pairs for each of the 608
+// schedulers. Below that a scheduler's one warp of pairs runs longer than its two warps of
+// single nodes (us a step from a graph, one node / pairs: 16 x 32 x 32 2.08 /
+// 2.59, 32^3 2.34 / 2.71, 128 x 128 x 5 3.36 / 3.30 and
+// 4.13 / 4.18 launched one by one, 48^3 4.06 / 3.36, 64^3
+// 6.27 / 5.41, 80^3 13.5 / 9.2, 150 x 91 x 61 with a force field 22.5 / 20.6,
+// 200 x 180 x 160 137 / 128, 256^3 371 / 362).
+bool step_pairs(const Geom &g) {
+    const int64_t npx = (g.nx + 1) / 2;
+    // the row of a pair by one multiplication: exact while pairs of a plane x pairs of a row < 2^32
+    return npx >= 2 && npx * npx * g.ny < ((int64_t)1 << 32) && (int64_t)g.nx * g.ny * g.nz >= 100000;
+}
+
+template <int FM>
+static cudaError_t pair_t(const Launch &L, const float *src, float *dst, const Rates &r, const ForceArgs &F,
+                          int *flag) {
+    const Geom &g = L.g;
+    const uint32_t npx = (uint32_t)(g.nx + 1) / 2u, rdiv = 0xffffffffu / npx + 1u;
+    const dim3 grid((npx * (uint32_t)g.ny + kPairThreads - 1u) / kPairThreads, (unsigned)g.nz);
+    const bool vec = g.nx % 2 == 0 && (((uintptr_t)src | (uintptr_t)dst) & 7u) == 0;
+    auto go = [&](auto kern) {
+        return launch_overlapped(kern, grid, dim3(kPairThreads), 0, L.stream, L.overlap, src, dst, g, r, F, flag, npx,
+                                 rdiv);
+    };
+    if (g.walls) return vec ? go(k_step_pair<FM, true, true>) : go(k_step_pair<FM, true, false>);
+    return vec ? go(k_step_pair<FM, false, true>) : go(k_step_pair<FM, false, false>);
+}
+
+cudaError_t launch_step_pair(const Launch &L, const void *src, void *dst, const Rates &r, const ForceArgs &F,
+                             int *flag) {
+    const float *s = (const float *)src;
+    float *d = (float *)dst;
+    switch (F.mode) {
+        case kForceUniform: return pair_t<kForceUniform>(L, s, d, r, F, flag);
+        case kForceProfileZ: return pair_t<kForceProfileZ>(L, s, d, r, F, flag);
+        default: return pair_t<kForceField>(L, s, d, r, F, flag);
+    }
+}
+
+}  // namespace clbm

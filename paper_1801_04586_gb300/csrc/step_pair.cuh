@@ -1,0 +1,117 @@
+// step_pair.cuh -- the FP32 D3Q19 A/B step with two adjacent nodes per thread,
+// collided together in the lanes of f2 (FP32x2 instructions).
+//
+// Why: with the populations in L2 (up to some 80^3) the one-node step is bound
+// by instruction issue and by the last wave of its blocks; above, it runs at
+// the DRAM rate only as long as enough of its warps are loading. A pair halves
+// the arithmetic's issue slots (f2 rounds like the one-node collision, so the
+// results are the same bits), forms each address once for two nodes and moves
+// 9 of 19 populations by 64-bit loads and all of them by 64-bit stores. 78-80
+// registers for the pair (96 and 88 with odd rows) keep six blocks of 128, 24
+// warps of pairs, in flight on an SM. 256^3: 362 us a step
+// against 371 (7.05 TB/s algorithmic, 1.04 of the copy rate); 80^3 in L2: 9.2
+// against 13.5.
+//
+// (A pass of two steps over a column kept in shared memory, which halves the
+// DRAM traffic, measured 38-45k MLUPS in six forms, no more than the single
+// step's 46.4k: 16 warps per SM do not hide its phases.)
+#pragma once
+
+#include "cascaded.cuh"
+#include "kernels.cuh"
+#include "step_kernels.cuh"
+
+namespace clbm {
+
+constexpr int kPairThreads = 128;
+
+// The wall faces a node touches, and whether population i arrives from beyond
+// one of them (halfway bounce-back).
+struct WallFaces {
+    bool xl, xh, yl, yh, zl, zh;
+    __device__ __forceinline__ bool any() const { return xl || xh || yl || yh || zl || zh; }
+    __device__ __forceinline__ bool bounces(int i) const {
+        return (ex19(i) > 0 && xl) || (ex19(i) < 0 && xh) || (ey19(i) > 0 && yl) || (ey19(i) < 0 && yh) ||
+               (ez19(i) > 0 && zl) || (ez19(i) < 0 && zh);
+    }
+};
+__device__ __forceinline__ WallFaces wall_faces(const Geom &g, int x, int y, int z) {
+    const bool wx = g.walls & 1u, wy = g.walls & 2u, wz = g.walls & 4u;
+    return WallFaces{wx && x == 0, wx && x == g.nx - 1, wy && y == 0, wy && y == g.ny - 1, wz && z == 0,
+                     wz && z == g.nz - 1};
+}
+
+__device__ __forceinline__ float2 ld_state2(const float *p) {
+    float2 v;
+    asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+
+// VEC: nx even, so that a pair x, x + 1 (x even) is 8-byte aligned in every
+// row. Thread t of plane z takes pair t of the plane's rows of (nx + 1) / 2
+// pairs: no lane idles whatever nx is. rdiv = ceil(2^32 / pairs per row).
+template <int FM, bool WALLS, bool VEC>
+__global__ void __launch_bounds__(kPairThreads) k_step_pair(const float *src, float *__restrict__ dst, Geom g, Rates r,
+                                                            ForceArgs F, int *__restrict__ flag, uint32_t npx,
+                                                            uint32_t rdiv) {
+    grid_dependency_wait();
+    const uint32_t t = blockIdx.x * kPairThreads + threadIdx.x;
+    if (t >= npx * (uint32_t)g.ny) return;
+    const int y = (int)__umulhi(t, rdiv), z = blockIdx.y;
+    const int x = 2 * (int)(t - (uint32_t)y * npx);
+    const bool two = VEC || x + 1 < g.nx;
+    const uint32_t unx = (uint32_t)g.nx, plane = unx * (uint32_t)g.ny;
+    const uint32_t rc = (uint32_t)y * unx, rm = (uint32_t)(y == 0 ? g.ny - 1 : y - 1) * unx,
+                   rp = (uint32_t)(y == g.ny - 1 ? 0 : y + 1) * unx;
+    const uint32_t zc = (uint32_t)z * plane, zm = (uint32_t)(z == 0 ? g.nz - 1 : z - 1) * plane,
+                   zp = (uint32_t)(z == g.nz - 1 ? 0 : z + 1) * plane;
+    const uint32_t xa = (uint32_t)x, xb = two ? xa + 1u : xa;  // the pair (odd nx: a row's last pair is one node)
+    const uint32_t xam = xa == 0u ? unx - 1u : xa - 1u, xbp = xb == unx - 1u ? 0u : xb + 1u;
+    const uint32_t self = zc + rc + xa;
+    f2 h[kQ];
+#pragma unroll
+    for (int i = 0; i < kQ; ++i) {
+        const float *base = src + (size_t)i * g.stride;
+        const uint32_t row = (ez19(i) > 0 ? zm : (ez19(i) < 0 ? zp : zc)) + (ey19(i) > 0 ? rm : (ey19(i) < 0 ? rp : rc));
+        if (ex19(i) == 0 && VEC)
+            h[i] = f2{ld_state2(base + CLBM_IDX(g, row + xa))};
+        else if (ex19(i) == 0)
+            h[i] = mk2(ld_state(base + CLBM_IDX(g, row + xa)), ld_state(base + CLBM_IDX(g, row + xb)));
+        else if (ex19(i) > 0)
+            h[i] = mk2(ld_state(base + CLBM_IDX(g, row + xam)), ld_state(base + CLBM_IDX(g, row + (two ? xa : xam))));
+        else
+            h[i] = mk2(ld_state(base + CLBM_IDX(g, row + (two ? xb : xbp))), ld_state(base + CLBM_IDX(g, row + xbp)));
+    }
+    if (WALLS) {
+        const WallFaces wa = wall_faces(g, (int)xa, y, z), wb = wall_faces(g, (int)xb, y, z);
+        if (wa.any() || wb.any()) {
+#pragma unroll
+            for (int i = 1; i < kQ; ++i) {
+                const float *base = src + (size_t)opposite(i) * g.stride;
+                if (wa.bounces(i)) h[i].v.x = ld_state(base + CLBM_IDX(g, self));
+                if (wb.bounces(i)) h[i].v.y = ld_state(base + CLBM_IDX(g, self + (xb - xa)));
+            }
+        }
+    }
+    f2 fx, fy, fz;
+    {
+        float ax, ay, az;
+        force_at<FM>(F, g, z, self, ax, ay, az);
+        fx = mk2(ax); fy = mk2(ay); fz = mk2(az);
+        if (FM == kForceField) force_at<FM>(F, g, z, self + (xb - xa), fx.v.y, fy.v.y, fz.v.y);
+    }
+    const f2 drho = Cascaded::run<false>(h, fx, fy, fz, r);
+    if (!(fabsf(drho.v.x) < 0.9f) || !(fabsf(drho.v.y) < 0.9f)) *flag = 1;
+#pragma unroll
+    for (int i = 0; i < kQ; ++i) {
+        float *to = dst + (size_t)i * g.stride + CLBM_SLOTS(g, self, (kQ - 1) * g.stride + (xb - xa));
+        if (VEC) {
+            *reinterpret_cast<float2 *>(to) = h[i].v;
+        } else {
+            to[0] = h[i].v.x;
+            if (two) to[1] = h[i].v.y;
+        }
+    }
+}
+
+}  // namespace clbm
