@@ -112,8 +112,10 @@ extern "C" {
  *      and the cascaded D3Q19 in-place (AA) steps with 16-bit storage, stage
  *      the rows they read in shared memory with bulk asynchronous copies
  *      where the geometry allows (nx <= 1024, nx a multiple of 8; D3Q27 not
- *      with a force field); cascaded D3Q19 A/B steps with FP32 storage on
- *      lattices of 100,000 nodes or more collide two adjacent nodes per thread
+ *      with a force field) and the lattice is large enough for that to be the
+ *      faster form (400,000 to 1,500,000 nodes, see capi.cu; always if
+ *      wait_cycles is set); other cascaded D3Q19 A/B steps of lattices of
+ *      100,000 nodes or more collide two adjacent nodes per thread
  *      (unless block_x or block_y is given); one node per thread otherwise; 1: always one node per thread,
  *      plain loads (block_x, block_y apply); 2: two nodes per thread (x and
  *      x + block_x), collided together with the FP32x2 instructions (D3Q19
@@ -141,7 +143,8 @@ extern "C" {
  *      would. slab = 0 (the default) is an ordinary lattice. Slabs: D3Q19,
  *      cascaded model, A/B pattern, variant 0 (16-bit storage staged where it
  *      applies) or 1.
- * wait_cycles: bound, in SM clock cycles, of each wait of the staged step
+ * wait_cycles: (any value > 0 also makes every eligible step run staged,
+ *      whatever the lattice's size) bound, in SM clock cycles, of each wait of the staged step
  *      (variant 0, 16-bit storage) for the bulk copies of its next tile; 0
  *      selects 4e9 (about 2 s). A wait that runs out makes the kernel give up
  *      the step and return: every block first waits (bounded by 4e9 cycles)
@@ -191,7 +194,7 @@ typedef struct clbm_info {
     int32_t pattern;          /* CLBM_PATTERN_AB or CLBM_PATTERN_AA */
     int32_t buffers;          /* population buffers held: 2 (A/B) or 1 (AA) */
     int32_t model;            /* CLBM_MODEL_* */
-    int32_t staged;           /* 1: steps stage the pulled rows in shared memory (variant 0, see clbm_params) */
+    int32_t staged;           /* 1: steps can stage the pulled rows in shared memory (variant 0; small lattices do not, see clbm_params) */
     int32_t slab;             /* halo faces of a z-slab (clbm_params.slab) */
     int64_t face_bytes;       /* z-slab: bytes of one face's 5 populations (5 x nx x ny values), else 0 */
 } clbm_info;

@@ -86,8 +86,9 @@ struct clbm_ctx {
     int64_t steps_done;
     double gamma;         // force decay rate (clbm_set_force_decay)
     bool packed;          // step kernel with two nodes per thread (FP32x2 arithmetic)
-    bool pairs;           // FP32 steps with two adjacent nodes per thread (step_pair.cu)
-    bool staged;          // steps with rows staged in shared memory by bulk copies (variant 0; see clbm_create)
+    bool pairs;           // steps with two adjacent nodes per thread where they are not staged (step_pair.cu)
+    bool staged;          // steps with rows staged in shared memory by bulk copies apply (variant 0; see clbm_create)
+    bool run_staged;      // ... and the lattice is large enough for them to pay
     int q;                // 19 (Appendix A) or 27 (Sec. II)
     bool aa;              // in-place (AA) pattern: one population buffer, step kind by parity
     int model;            // CLBM_MODEL_*
@@ -153,7 +154,7 @@ Launch launch_of(const clbm_ctx *c) {
     L.grid = dim3((c->g.nx + c->block.x - 1) / c->block.x, (c->g.ny + c->block.y - 1) / c->block.y, c->g.nz);
     L.stream = c->stream;
     L.packed = false;
-    L.staged = c->staged;
+    L.staged = c->run_staged;
     L.pairs = c->pairs;
     // A/B: the pull map (through the halo planes for a z-slab); AA: natural
     // slots after an even number of steps, the odd step's swapped pull map
@@ -172,6 +173,34 @@ Launch step_launch_of(const clbm_ctx *c) {
         L.grid.x = (c->g.nx + 2 * c->block.x - 1) / (2 * c->block.x);
     }
     return L;
+}
+
+// The smallest lattice whose 16-bit steps run staged. A staged block works
+// through tiles of 768-1024 nodes, so a small lattice leaves most SMs idle and
+// the rest with one tile's copy latency and nothing behind it. Measured (us a
+// step, staged / the form that replaces it):
+//   A/B cascaded against node pairs: FP16 48^3 4.9 / 3.0, 80^3 10.3 / 9.2,
+//     104^3 20.4 / 18.0, 128^3 34.4 / 36.9, 256^3 228 / 271; FP16-SR 48^3
+//     6.8 / 4.3, 104^3 22.4 / 19.0, 128^3 37.3 / 37.9, 256^3 251 / 278;
+//     against one node per thread (below 100,000 nodes) 32^3 6.1 / 2.2;
+//   A/B SRT and MRT against one node: 64^3 6.7 / 5.8, 96^3 17.5 / 15.7, 128^3
+//     36.4 / 36.8;
+//   in place against one node: FP16 32^3 4.9 / 2.2, 64^3 6.8 / 6.3, 80^3 11.0
+//     / 12.6; FP16-SR 64^3 7.7 / 7.5, 80^3 12.0 / 15.3;
+//   D3Q27 against one node: FP16 32^3 7.2 / 2.8, 64^3 10.2 / 9.5 (walls 17.4 /
+//     10.2), 80^3 17.8 / 20.2, 128^3 62 / 64; stochastic rounding 64^3 13.1 /
+//     11.2, 128^3 80 / 78, 160^3 159 / 152: one node at every size.
+// A context that bounds or injects the staged waits runs them at any size, as
+// do z-slabs (not measured across GPUs) and the bounds-checked build.
+int64_t staged_min_nodes(const clbm_params &p, int q, bool pairs) {
+#ifdef CLBM_BOUNDS_CHECK
+    return 0;
+#endif
+    if (p.slab || p.inject || p.wait_cycles > 0) return 0;
+    const bool stochastic = p.storage == CLBM_STORAGE_F16_SR || p.storage == CLBM_STORAGE_BF16_SR;
+    if (q == 27) return stochastic ? INT64_MAX : 400000;
+    if (p.pattern == CLBM_PATTERN_AA) return 400000;
+    return pairs || p.model != CLBM_MODEL_CASCADED ? 1500000 : 250000;
 }
 
 bool rate_ok(double s) { return std::isfinite(s) && s > 0.0 && s < 2.0; }
@@ -356,12 +385,13 @@ int clbm_create(const clbm_params *p, void *stream, clbm_ctx **out) {
     c->gamma = 0.0;
     c->q = q;
     c->packed = q == 19 && p->variant == 2;
-    // staged: A/B steps, and the cascaded D3Q19 in-place step (node pairs)
+    // pairs: A/B cascaded D3Q19 steps that are not staged, unless the caller chose a block of the one-node kernel
+    c->pairs = q == 19 && p->variant == 0 && p->pattern == CLBM_PATTERN_AB && p->model == CLBM_MODEL_CASCADED &&
+               !p->slab && p->block_x == 0 && p->block_y == 0 && step_pairs(c->g);
+    // staged: A/B steps, and the cascaded D3Q19 in-place step (node pairs); they run so from staged_min_nodes on
     c->staged = p->variant == 0 &&
                 (p->pattern != CLBM_PATTERN_AA || (q == 19 && p->model == CLBM_MODEL_CASCADED));
-    // pairs: FP32 A/B cascaded D3Q19 steps, unless the caller chose a block shape of the one-node kernel
-    c->pairs = q == 19 && p->variant == 0 && p->storage == CLBM_STORAGE_F32 && p->pattern == CLBM_PATTERN_AB &&
-               p->model == CLBM_MODEL_CASCADED && !p->slab && p->block_x == 0 && p->block_y == 0 && step_pairs(c->g);
+    c->run_staged = c->staged && n >= staged_min_nodes(*p, q, c->pairs);
     c->aa = p->pattern == CLBM_PATTERN_AA;
     c->model = p->model;
     c->rates27.om2 = c->rates.om2;

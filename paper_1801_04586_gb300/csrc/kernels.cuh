@@ -79,7 +79,7 @@ struct Launch {
     dim3 block, grid;  // grid of the one-node-per-thread kernels
     cudaStream_t stream;
     bool overlap = true;  // launch_overlapped: not inside a graph capture
-    bool pairs = false;   // launch_step, FP32: two adjacent nodes per thread (step_pair.cu)
+    bool pairs = false;   // launch_step, where the staged form does not apply: two adjacent nodes per thread (step_pair.cu)
     bool packed;       // launch_step: two nodes per thread (grid.x halved)
     bool staged;       // launch_step (A/B) and launch_step_aa (16-bit, cascaded): rows staged by bulk copies
                        // where they apply (step_tma.cuh)
@@ -96,12 +96,12 @@ struct Launch {
 // (CLBM_STORAGE_*). key: per-step dither key (stochastic formats).
 cudaError_t launch_step(int storage, const Launch &L, const void *src, void *dst, const Rates &r,
                         const ForceArgs &F, int *flag, uint32_t key);
-// One cascaded FP32 step with two adjacent nodes per thread (step_pair.cu):
+// One cascaded A/B step with two adjacent nodes per thread (step_pair.cu):
 // whether a lattice takes it by default, and its launch (the bits of
 // launch_step's one-node kernel).
 bool step_pairs(const Geom &g);
-cudaError_t launch_step_pair(const Launch &L, const void *src, void *dst, const Rates &r, const ForceArgs &F,
-                             int *flag);
+cudaError_t launch_step_pair(int storage, const Launch &L, const void *src, void *dst, const Rates &r,
+                             const ForceArgs &F, int *flag, uint32_t key);
 // The cascaded step on a z-slab (Geom::slab halo faces): the planes z0,
 // z0 + zs, ... (nplanes of them) from src into dst (step.cu).
 cudaError_t launch_step_slab(int storage, const Launch &L, const void *src, void *dst, const Rates &r,

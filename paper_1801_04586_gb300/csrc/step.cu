@@ -70,7 +70,8 @@ static cudaError_t step2_force(const Launch &L, const void *src, void *dst, cons
 
 cudaError_t launch_step(int storage, const Launch &L, const void *src, void *dst, const Rates &r,
                         const ForceArgs &F, int *flag, uint32_t key) {
-    if (L.pairs && storage == 0) return launch_step_pair(L, src, dst, r, F, flag);
+    if (L.pairs && !(L.staged && step_staged(L.g, storage == 0 ? 4 : 2, src, 19, F.mode)))
+        return launch_step_pair(storage, L, src, dst, r, F, flag, key);
     if (!L.packed) return launch_step_with<Cascaded>(storage, L, src, dst, r, F, flag, key);
     switch (storage) {
         case 0: return step2_force<float>(L, src, dst, r, F, flag, key);

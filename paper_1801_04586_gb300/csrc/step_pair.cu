@@ -16,29 +16,44 @@ bool step_pairs(const Geom &g) {
     return npx >= 2 && npx * npx * g.ny < ((int64_t)1 << 32) && (int64_t)g.nx * g.ny * g.nz >= 100000;
 }
 
-template <int FM>
-static cudaError_t pair_t(const Launch &L, const float *src, float *dst, const Rates &r, const ForceArgs &F,
-                          int *flag) {
+template <typename S, int FM>
+static cudaError_t pair_t(const Launch &L, const void *src, void *dst, const Rates &r, const ForceArgs &F, int *flag,
+                          uint32_t key) {
     const Geom &g = L.g;
     const uint32_t npx = (uint32_t)(g.nx + 1) / 2u, rdiv = 0xffffffffu / npx + 1u;
     const dim3 grid((npx * (uint32_t)g.ny + kPairThreads - 1u) / kPairThreads, (unsigned)g.nz);
-    const bool vec = g.nx % 2 == 0 && (((uintptr_t)src | (uintptr_t)dst) & 7u) == 0;
-    auto go = [&](auto kern) {
-        return launch_overlapped(kern, grid, dim3(kPairThreads), 0, L.stream, L.overlap, src, dst, g, r, F, flag, npx,
-                                 rdiv);
+    const bool vec = g.nx % 2 == 0 && (((uintptr_t)src | (uintptr_t)dst) & (2 * sizeof(S) - 1u)) == 0;
+    auto go = [&](auto kern, auto... keys) {
+        return launch_overlapped(kern, grid, dim3(kPairThreads), 0, L.stream, L.overlap, (const S *)src, (S *)dst, g, r,
+                                 F, flag, keys..., npx, rdiv);
     };
-    if (g.walls) return vec ? go(k_step_pair<FM, true, true>) : go(k_step_pair<FM, true, false>);
-    return vec ? go(k_step_pair<FM, false, true>) : go(k_step_pair<FM, false, false>);
+    if constexpr (sizeof(S) == 4) {
+        if (g.walls) return vec ? go(k_step_pair<FM, true, true>) : go(k_step_pair<FM, true, false>);
+        return vec ? go(k_step_pair<FM, false, true>) : go(k_step_pair<FM, false, false>);
+    } else {
+        if (g.walls) return vec ? go(k_step_pair16<S, FM, true, true>, key) : go(k_step_pair16<S, FM, true, false>, key);
+        return vec ? go(k_step_pair16<S, FM, false, true>, key) : go(k_step_pair16<S, FM, false, false>, key);
+    }
 }
 
-cudaError_t launch_step_pair(const Launch &L, const void *src, void *dst, const Rates &r, const ForceArgs &F,
-                             int *flag) {
-    const float *s = (const float *)src;
-    float *d = (float *)dst;
+template <typename S>
+static cudaError_t pair_force_t(const Launch &L, const void *src, void *dst, const Rates &r, const ForceArgs &F,
+                                int *flag, uint32_t key) {
     switch (F.mode) {
-        case kForceUniform: return pair_t<kForceUniform>(L, s, d, r, F, flag);
-        case kForceProfileZ: return pair_t<kForceProfileZ>(L, s, d, r, F, flag);
-        default: return pair_t<kForceField>(L, s, d, r, F, flag);
+        case kForceUniform: return pair_t<S, kForceUniform>(L, src, dst, r, F, flag, key);
+        case kForceProfileZ: return pair_t<S, kForceProfileZ>(L, src, dst, r, F, flag, key);
+        default: return pair_t<S, kForceField>(L, src, dst, r, F, flag, key);
+    }
+}
+
+cudaError_t launch_step_pair(int storage, const Launch &L, const void *src, void *dst, const Rates &r,
+                             const ForceArgs &F, int *flag, uint32_t key) {
+    switch (storage) {
+        case 0: return pair_force_t<float>(L, src, dst, r, F, flag, key);
+        case 1: return pair_force_t<__half>(L, src, dst, r, F, flag, key);
+        case 2: return pair_force_t<__nv_bfloat16>(L, src, dst, r, F, flag, key);
+        case 3: return pair_force_t<HalfSR>(L, src, dst, r, F, flag, key);
+        default: return pair_force_t<BF16SR>(L, src, dst, r, F, flag, key);
     }
 }
 

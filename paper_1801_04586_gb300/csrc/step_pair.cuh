@@ -1,4 +1,4 @@
-// step_pair.cuh -- the FP32 D3Q19 A/B step with two adjacent nodes per thread,
+// step_pair.cuh -- the D3Q19 A/B step with two adjacent nodes per thread,
 // collided together in the lanes of f2 (FP32x2 instructions).
 //
 // Why: with the populations in L2 (up to some 80^3) the one-node step is bound
@@ -41,13 +41,14 @@ __device__ __forceinline__ WallFaces wall_faces(const Geom &g, int x, int y, int
                      wz && z == g.nz - 1};
 }
 
+// An aligned pair of adjacent values (global memory, as ld_state).
 __device__ __forceinline__ float2 ld_state2(const float *p) {
     float2 v;
     asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
     return v;
 }
 
-// VEC: nx even, so that a pair x, x + 1 (x even) is 8-byte aligned in every
+// The FP32 step. VEC: nx even, so that a pair x, x + 1 (x even) is 8-byte aligned in every
 // row. Thread t of plane z takes pair t of the plane's rows of (nx + 1) / 2
 // pairs: no lane idles whatever nx is. rdiv = ceil(2^32 / pairs per row).
 template <int FM, bool WALLS, bool VEC>
@@ -112,6 +113,117 @@ __global__ void __launch_bounds__(kPairThreads) k_step_pair(const float *src, fl
             if (two) to[1] = h[i].v.y;
         }
     }
+}
+
+template <typename S>
+__device__ __forceinline__ float2 ld_state2(const S *p) {  // 16-bit formats: one word
+    uint32_t w;
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(w) : "l"(p));
+    return Codec<S>::unpack2(w);
+}
+
+// 16-bit formats: load what arrives at the nodes x and x + 1 (x even) of row y, plane z under
+// Eq. 8; returns the first one's offset. VEC: nx even, so that such a pair is
+// aligned in every row; otherwise two says whether x + 1 is a node (a row's
+// last pair of an odd row is one node: its second lane repeats the first).
+template <typename S, bool WALLS, bool VEC>
+__device__ __forceinline__ uint32_t pair_load(const S *src, const Geom &g, int x, int y, int z, bool two,
+                                              f2 (&h)[kQ]) {
+    const uint32_t unx = (uint32_t)g.nx, plane = unx * (uint32_t)g.ny;
+    const uint32_t rc = (uint32_t)y * unx, rm = (uint32_t)(y == 0 ? g.ny - 1 : y - 1) * unx,
+                   rp = (uint32_t)(y == g.ny - 1 ? 0 : y + 1) * unx;
+    const uint32_t zc = (uint32_t)z * plane, zm = (uint32_t)(z == 0 ? g.nz - 1 : z - 1) * plane,
+                   zp = (uint32_t)(z == g.nz - 1 ? 0 : z + 1) * plane;
+    const uint32_t xa = (uint32_t)x, xb = two ? xa + 1u : xa;
+    const uint32_t xam = xa == 0u ? unx - 1u : xa - 1u, xbp = xb == unx - 1u ? 0u : xb + 1u;
+    const uint32_t self = zc + rc + xa;
+#pragma unroll
+    for (int i = 0; i < kQ; ++i) {
+        const size_t pop = (size_t)i * g.stride;
+        const uint32_t row = (ez19(i) > 0 ? zm : (ez19(i) < 0 ? zp : zc)) + (ey19(i) > 0 ? rm : (ey19(i) < 0 ? rp : rc));
+        if (ex19(i) == 0 && VEC) {
+            h[i] = f2{ld_state2(src + CLBM_IDX(g, pop + (row + xa)))};
+        } else {
+            const uint32_t oa = row + (ex19(i) > 0 ? xam : (ex19(i) < 0 ? (two ? xb : xbp) : xa));
+            const uint32_t ob = row + (ex19(i) > 0 ? (two ? xa : xam) : (ex19(i) < 0 ? xbp : xb));
+            h[i] = mk2(Codec<S>::load(src + CLBM_IDX(g, pop + oa)), Codec<S>::load(src + CLBM_IDX(g, pop + ob)));
+        }
+    }
+    if (WALLS) {
+        const WallFaces wa = wall_faces(g, (int)xa, y, z), wb = wall_faces(g, (int)xb, y, z);
+        if (wa.any() || wb.any()) {
+#pragma unroll
+            for (int i = 1; i < kQ; ++i) {
+                const size_t b = (size_t)opposite(i) * g.stride + self;
+                if (wa.bounces(i)) h[i].v.x = Codec<S>::load(src + CLBM_IDX(g, b));
+                if (wb.bounces(i)) h[i].v.y = Codec<S>::load(src + CLBM_IDX(g, b + (xb - xa)));
+            }
+        }
+    }
+    return self;
+}
+
+// Store the pair's post-collision values at its own slots: a pair of an even
+// row is one conversion and one word; in odd rows each node converts on its own (the dither is drawn per even-odd pair of node indices).
+template <typename S, bool VEC>
+__device__ __forceinline__ void pair_store(S *dst, const Geom &g, uint32_t self, bool two, const f2 (&h)[kQ],
+                                           uint32_t key) {
+    S *at = dst + CLBM_SLOTS(g, self, (kQ - 1) * g.stride + (two ? 1u : 0u));
+    if constexpr (VEC) {
+        const uint32_t hb = Codec<S>::kStochastic ? pair_hash(self >> 1, key) : 0u;
+#pragma unroll
+        for (int i = 0; i < kQ; ++i) {
+            uint32_t w;
+            if constexpr (Codec<S>::kStochastic)
+                w = Codec<S>::pair_sr(h[i].v.y, h[i].v.x, pop_bits(hb, i));
+            else
+                w = Codec<S>::pair_rn(h[i].v.y, h[i].v.x);
+            *reinterpret_cast<uint32_t *>(at + (size_t)i * g.stride) = w;
+        }
+    } else {
+        const uint32_t ha = Codec<S>::kStochastic ? pair_hash(self >> 1, key) : 0u;
+        const uint32_t hb = Codec<S>::kStochastic ? pair_hash((self + 1u) >> 1, key) : 0u;
+#pragma unroll
+        for (int i = 0; i < kQ; ++i) {
+            S *to = at + (size_t)i * g.stride;
+            if constexpr (Codec<S>::kStochastic) {
+                to[0] = Codec<S>::from_f_sr(h[i].v.x, pop_bits(ha, i), self & 1u);
+                if (two) to[1] = Codec<S>::from_f_sr(h[i].v.y, pop_bits(hb, i), (self + 1u) & 1u);
+            } else {
+                to[0] = Codec<S>::from_f(h[i].v.x);
+                if (two) to[1] = Codec<S>::from_f(h[i].v.y);
+            }
+        }
+    }
+}
+
+// The 16-bit A/B step in node pairs, for lattices that the staged step
+// (step_tma.cuh) does not take or does not pay for. Without walls the pair is
+// capped at five blocks of 128 per SM (96 registers): FP16 at 151 x 90 x 61
+// 17.3 -> 14.5 us a step (17.6 one node per thread); with walls it keeps its
+// 104-122 registers (150 x 91 x 61: 15.0 us, 15.4 capped, 19.9 one node).
+template <typename S, int FM, bool WALLS, bool VEC>
+__global__ void __launch_bounds__(kPairThreads, WALLS ? 1 : 5)
+    k_step_pair16(const S *src, S *__restrict__ dst, Geom g, Rates r, ForceArgs F, int *__restrict__ flag,
+                  uint32_t key, uint32_t npx, uint32_t rdiv) {
+    grid_dependency_wait();
+    const uint32_t t = blockIdx.x * kPairThreads + threadIdx.x;
+    if (t >= npx * (uint32_t)g.ny) return;
+    const int y = (int)__umulhi(t, rdiv), z = blockIdx.y;
+    const int x = 2 * (int)(t - (uint32_t)y * npx);
+    const bool two = VEC || x + 1 < g.nx;
+    f2 h[kQ];
+    const uint32_t self = pair_load<S, WALLS, VEC>(src, g, x, y, z, two, h);
+    f2 fx, fy, fz;
+    {
+        float ax, ay, az;
+        force_at<FM>(F, g, z, self, ax, ay, az);
+        fx = mk2(ax); fy = mk2(ay); fz = mk2(az);
+        if (FM == kForceField) force_at<FM>(F, g, z, self + (two ? 1u : 0u), fx.v.y, fy.v.y, fz.v.y);
+    }
+    const f2 drho = Cascaded::run<true>(h, fx, fy, fz, r);
+    if (!(fabsf(drho.v.x) < 0.9f) || !(fabsf(drho.v.y) < 0.9f)) *flag = 1;
+    pair_store<S, VEC>(dst, g, self, two, h, key);
 }
 
 }  // namespace clbm
