@@ -6,8 +6,8 @@
 // kernel (pull, Eqs. 5, 7, 8, 9 in deviation form; see d3q19.cuh). The
 // domains' populations share two A/B allocations, domain after domain, each in
 // the single-lattice layout. A host-built work list cuts every domain into
-// tiles of T consecutive nodes in its linear index (T = threads per block),
-// so every lane has a node whatever the domain's extents, a warp reads
+// tiles of T consecutive nodes in its linear index (T = threads per block;
+// pairs of nodes with 16-bit storage), so every lane has a node whatever the domain's extents, a warp reads
 // contiguous memory, and only a domain's last tile is partial. A grid of
 // (SMs x resident blocks) walks the list with a stride: one launch covers all
 // domains. Steps are replayed from a captured CUDA graph.
@@ -22,6 +22,7 @@
 
 #include "../../include/clbm.h"
 #include "kernels.cuh"
+#include "step_pair.cuh"
 
 using namespace clbm;
 
@@ -62,12 +63,24 @@ struct DomainDesc {
     Rates r;
     float fx, fy, fz;
     float inv_nx, inv_ny;  // 1/nx, 1/ny (FP32) for the tile coordinate decode
+    float inv_npx;         // 1/npx, npx = (nx + 1) / 2 node pairs per row
     int64_t offset;        // element offset of the domain's 19 x stride block in A and in B
 };
 
+// Nodes per thread of the A/B kernel: 16-bit formats take pairs of adjacent
+// nodes (step_pair.cuh), FP32 one node. The FP32 batch runs near the DRAM rate
+// on 64 registers, which a pair does not reach (us a step of the benchmark's 64
+// domains: one node 808-818, pairs 876 at 108 registers, 1112 capped at 80);
+// the 16-bit batch is bound by instruction issue (FP16: 707-729 one node, 602
+// pairs).
+template <typename S>
+constexpr int kBatchNodes = sizeof(S) == 2 ? 2 : 1;
+
 // SMEM: the domain table is staged in shared memory once per launch (the
 // usual case); otherwise it is read through the read-only cache. The next
-// tile's entry is fetched while the current tile is processed.
+// tile's entry is fetched while the current tile is processed. A tile is
+// blockDim.x consecutive nodes of the domain, or pairs of adjacent nodes in
+// the order of rows of (nx + 1) / 2 pairs, one per thread.
 template <typename S, bool SMEM>
 __global__ void __launch_bounds__(512) k_batch_step(const S *A, S *__restrict__ B,
                                                     const DomainDesc *__restrict__ doms, int ndom,
@@ -81,27 +94,41 @@ __global__ void __launch_bounds__(512) k_batch_step(const S *A, S *__restrict__ 
     grid_dependency_wait();  // (the domain table and the work list stay unchanged while steps run)
     int t = blockIdx.x;
     if (t >= ntiles) return;
-    int4 tile = __ldg(tiles + t);  // (domain, x, y, z) of the tile's first node
+    int4 tile = __ldg(tiles + t);  // (domain, x or pair of the row, y, z) of the tile's first node or pair
     for (; t < ntiles; t += gridDim.x) {
         const int tn = t + gridDim.x;
         const int4 next = tn < ntiles ? __ldg(tiles + tn) : tile;
         const DomainDesc *D = SMEM ? sdom + tile.x : doms + tile.x;
         const Geom g = D->g;
-        // node tile_start + threadIdx.x: carry x into y and y into z. The
+        // entry tile_start + threadIdx.x: carry x into y and y into z. The
         // quotients are below 2^17, so floor((v + 0.5) * (1/n)) in FP32 is exact.
+        const int row = kBatchNodes<S> == 2 ? (g.nx + 1) >> 1 : g.nx;
         const int xt = tile.y + (int)threadIdx.x;
-        const int cy = (int)(((float)xt + 0.5f) * D->inv_nx);
+        const int cy = (int)(((float)xt + 0.5f) * (kBatchNodes<S> == 2 ? D->inv_npx : D->inv_nx));
         const int yt = tile.z + cy;
         const int cz = (int)(((float)yt + 0.5f) * D->inv_ny);
-        const int x = xt - cy * g.nx, y = yt - cz * g.ny, z = tile.w + cz;
+        const int x = kBatchNodes<S> * (xt - cy * row), y = yt - cz * g.ny, z = tile.w + cz;
         if (z < g.nz) {
             const S *src = A + D->offset;
             S *dst = B + D->offset;
-            float h[kQ];
-            const uint32_t self = pull_load<S, true>(src, g, x, y, z, h);
-            const float drho = collide<sizeof(S) == 2>(h, D->fx, D->fy, D->fz, D->r);
-            if (!(fabsf(drho) < 0.9f)) *flag = 1;
-            store_node<S>(dst + self, g.stride, h, self, 0u);
+            if constexpr (kBatchNodes<S> == 2) {
+                const bool even = (g.nx & 1) == 0, two = x + 1 < g.nx;
+                f2 h[kQ];
+                const uint32_t self = even ? pair_load<S, true, true>(src, g, x, y, z, true, h)
+                                           : pair_load<S, true, false>(src, g, x, y, z, two, h);
+                const f2 drho = collide<true>(h, mk2(D->fx), mk2(D->fy), mk2(D->fz), D->r);
+                if (!(fabsf(drho.v.x) < 0.9f) || !(fabsf(drho.v.y) < 0.9f)) *flag = 1;
+                if (even)
+                    pair_store<S, true>(dst, g, self, true, h, 0u);
+                else
+                    pair_store<S, false>(dst, g, self, two, h, 0u);
+            } else {
+                float h[kQ];
+                const uint32_t self = pull_load<S, true>(src, g, x, y, z, h);
+                const float drho = collide<false>(h, D->fx, D->fy, D->fz, D->r);
+                if (!(fabsf(drho) < 0.9f)) *flag = 1;
+                store_node<S>(dst + self, g.stride, h, self, 0u);
+            }
         }
         tile = next;
     }
@@ -174,15 +201,10 @@ constexpr int kSmemDomains = 512;  // domain tables up to this size are staged i
 
 template <typename S>
 static cudaError_t batch_launch_t(const void *A, void *B, const DomainDesc *doms, int ndom, const int4 *tiles,
-                                  int ntiles, int grid, dim3 block, int *flag, cudaStream_t s,
-                                bool overlap) {
-    if (ndom <= kSmemDomains)
-        launch_overlapped(k_batch_step<S, true>, grid, block, sizeof(DomainDesc) * ndom, s, overlap, (const S *)A,
-                          (S *)B, doms, ndom, tiles, ntiles, flag);
-    else
-        launch_overlapped(k_batch_step<S, false>, grid, block, 0, s, overlap, (const S *)A, (S *)B, doms, ndom,
-                          tiles, ntiles, flag);
-    return cudaGetLastError();
+                                  int ntiles, int grid, dim3 block, int *flag, cudaStream_t s, bool overlap) {
+    const size_t sm = ndom <= kSmemDomains ? sizeof(DomainDesc) * ndom : 0;
+    return launch_overlapped(ndom <= kSmemDomains ? k_batch_step<S, true> : k_batch_step<S, false>, grid, block, sm, s,
+                             overlap, (const S *)A, (S *)B, doms, ndom, tiles, ntiles, flag);
 }
 
 template <typename S>
@@ -227,12 +249,9 @@ static cudaError_t batch_launch(int storage, const void *A, void *B, const Domai
 template <typename S>
 static int occupancy_t(int threads, int ndom) {
     int per_sm = 0;
-    cudaError_t e;
-    if (ndom <= kSmemDomains)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch_step<S, true>, threads,
-                                                          sizeof(DomainDesc) * ndom);
-    else
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_batch_step<S, false>, threads, 0);
+    const size_t sm = ndom <= kSmemDomains ? sizeof(DomainDesc) * ndom : 0;
+    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+        &per_sm, ndom <= kSmemDomains ? k_batch_step<S, true> : k_batch_step<S, false>, threads, sm);
     return (e == cudaSuccess && per_sm > 0) ? per_sm : 1;
 }
 
@@ -307,15 +326,17 @@ void *domain_ptr(const clbm_batch *b, int which, int d) {
 }
 
 // Build and upload the work list for T threads per block: tiles of T
-// consecutive linear nodes, domain after domain.
+// consecutive nodes, or pairs of nodes (kBatchNodes), domain after domain.
 int build_tiles(clbm_batch *b, int T) {
     std::vector<int4> tiles;
     for (int d = 0; d < b->ndom; ++d) {
         const Geom &g = b->descs[d].g;
-        const int64_t n = (int64_t)g.nx * g.ny * g.nz;
+        const bool pairs = !b->aa && b->storage != CLBM_STORAGE_F32;  // kBatchNodes
+        const int64_t row = pairs ? (g.nx + 1) / 2 : g.nx;
+        const int64_t n = row * g.ny * g.nz;
         for (int64_t s0 = 0; s0 < n; s0 += T) {
-            const int x = (int)(s0 % g.nx);
-            const int64_t r = s0 / g.nx;
+            const int x = (int)(s0 % row);
+            const int64_t r = s0 / row;
             tiles.push_back(make_int4(d, x, (int)(r % g.ny), (int)(r / g.ny)));
         }
     }
@@ -431,6 +452,7 @@ int clbm_batch_create_pattern(const clbm_domain *doms, int32_t ndomains, int32_t
         D.fx = (float)p.fx; D.fy = (float)p.fy; D.fz = (float)p.fz;
         D.inv_nx = 1.0f / (float)p.nx;
         D.inv_ny = 1.0f / (float)p.ny;
+        D.inv_npx = 1.0f / (float)((p.nx + 1) / 2);
         D.offset = off;
         off += (int64_t)kQ * D.g.stride;
         nodes += n;
