@@ -187,9 +187,9 @@ Launch step_launch_of(const clbm_ctx *c) {
 //     36.4 / 36.8;
 //   in place against one node: FP16 32^3 4.9 / 2.2, 64^3 6.8 / 6.3, 80^3 11.0
 //     / 12.6; FP16-SR 64^3 7.7 / 7.5, 80^3 12.0 / 15.3;
-//   D3Q27 against one node: FP16 32^3 7.2 / 2.8, 64^3 10.2 / 9.5 (walls 17.4 /
-//     10.2), 80^3 17.8 / 20.2, 128^3 62 / 64; stochastic rounding 64^3 13.1 /
-//     11.2, 128^3 80 / 78, 160^3 159 / 152: one node at every size.
+//   D3Q27 against one node: FP16 80^3 15.6 / 20.2, 128^3 56 / 64; FP16-SR 80^3
+//     16.2 / 24.4, 128^3 58 / 78; one tile per plane and SM below that (32^3
+//     7.2 / 2.8 and 64^3 with walls 17.4 / 10.2 in the one-node staged form).
 // A context that bounds or injects the staged waits runs them at any size, as
 // do z-slabs (not measured across GPUs) and the bounds-checked build.
 int64_t staged_min_nodes(const clbm_params &p, int q, bool pairs) {
@@ -197,9 +197,7 @@ int64_t staged_min_nodes(const clbm_params &p, int q, bool pairs) {
     return 0;
 #endif
     if (p.slab || p.inject || p.wait_cycles > 0) return 0;
-    const bool stochastic = p.storage == CLBM_STORAGE_F16_SR || p.storage == CLBM_STORAGE_BF16_SR;
-    if (q == 27) return stochastic ? INT64_MAX : 400000;
-    if (p.pattern == CLBM_PATTERN_AA) return 400000;
+    if (q == 27 || p.pattern == CLBM_PATTERN_AA) return 400000;
     return pairs || p.model != CLBM_MODEL_CASCADED ? 1500000 : 250000;
 }
 

@@ -473,6 +473,23 @@ using ::fmaf;
 __device__ __forceinline__ f2 fmaf(f2 a, f2 b, f2 c) { return f2{__ffma2_rn(a.v, b.v, c.v)}; }
 __device__ __forceinline__ f2 fmaf(float a, f2 b, f2 c) { return fmaf(mk2(a), b, c); }
 
+// A constant in the type of a value.
+__device__ __forceinline__ float mk_like(float, float a) { return a; }
+__device__ __forceinline__ f1 mk_like(f1, float a) { return mk1(a); }
+__device__ __forceinline__ f2 mk_like(f2, float a) { return mk2(a); }
+
+// Make values opaque: the compiler must treat them as new from here on.
+__device__ __forceinline__ void hide1(float &a) { asm volatile("" : "+f"(a)); }
+__device__ __forceinline__ void hide1(f1 &a) { hide1(a.v); }
+__device__ __forceinline__ void hide1(f2 &a) {
+    hide1(a.v.x);
+    hide1(a.v.y);
+}
+template <typename... T>
+__device__ __forceinline__ void hide(T &...a) {
+    (hide1(a), ...);
+}
+
 // 1/x for x near 1 (the density): the hardware reciprocal estimate
 // (rcp.approx, relative error below 2^-23) refined by one Newton-Raphson
 // step, e = 1 - x r, r' = r + r e, which leaves it within an ulp of the

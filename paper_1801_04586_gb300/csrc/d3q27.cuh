@@ -89,38 +89,40 @@ __device__ __forceinline__ void pull_sources27(const Geom &g, int x, int y, int 
 // Per-axis transforms on a cube. Axis A, line (i, j) over the other two axes.
 #define CLBM_CUBE_LINE(c, A, i, j, k) (A == 0 ? c[k][i][j] : (A == 1 ? c[i][k][j] : c[i][j][k]))
 
-template <int A>
-__device__ __forceinline__ void raw_axis(float (&c)[3][3][3]) {
+template <int A, typename T>
+__device__ __forceinline__ void raw_axis(T (&c)[3][3][3]) {
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-            float &f0 = CLBM_CUBE_LINE(c, A, i, j, 0), &fp = CLBM_CUBE_LINE(c, A, i, j, 1),
-                  &fm = CLBM_CUBE_LINE(c, A, i, j, 2);
-            const float k2 = fp + fm, k1 = fp - fm;
+            T &f0 = CLBM_CUBE_LINE(c, A, i, j, 0), &fp = CLBM_CUBE_LINE(c, A, i, j, 1),
+              &fm = CLBM_CUBE_LINE(c, A, i, j, 2);
+            const T k2 = fp + fm, k1 = fp - fm;
             f0 = f0 + k2;
             fp = k1;
             fm = k2;
         }
 }
 
-template <int A>
-__device__ __forceinline__ void inverse_axis(float (&c)[3][3][3]) {
+// (k2 + k1)/2 and (k2 - k1)/2 as k2/2 +- k1/2, whose halves are exact: the
+// same bits with one multiply fewer.
+template <int A, typename T>
+__device__ __forceinline__ void inverse_axis(T (&c)[3][3][3]) {
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-            float &k0 = CLBM_CUBE_LINE(c, A, i, j, 0), &k1 = CLBM_CUBE_LINE(c, A, i, j, 1),
-                  &k2 = CLBM_CUBE_LINE(c, A, i, j, 2);
-            const float fp = 0.5f * (k2 + k1), fm = 0.5f * (k2 - k1);
+            T &k0 = CLBM_CUBE_LINE(c, A, i, j, 0), &k1 = CLBM_CUBE_LINE(c, A, i, j, 1),
+              &k2 = CLBM_CUBE_LINE(c, A, i, j, 2);
+            const T half = 0.5f * k2, fp = fmaf(0.5f, k1, half), fm = fmaf(-0.5f, k1, half);
             k0 = k0 - k2;
             k1 = fp;
             k2 = fm;
         }
 }
 
-template <int A>
-__device__ __forceinline__ void shift_axis(float (&c)[3][3][3], float v) {
+template <int A, typename T>
+__device__ __forceinline__ void shift_axis(T (&c)[3][3][3], T v) {
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
@@ -128,8 +130,8 @@ __device__ __forceinline__ void shift_axis(float (&c)[3][3][3], float v) {
             shift3(CLBM_CUBE_LINE(c, A, i, j, 0), CLBM_CUBE_LINE(c, A, i, j, 1), CLBM_CUBE_LINE(c, A, i, j, 2), v);
 }
 
-template <int A>
-__device__ __forceinline__ void unshift_axis(float (&c)[3][3][3], float v) {
+template <int A, typename T>
+__device__ __forceinline__ void unshift_axis(T (&c)[3][3][3], T v) {
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
@@ -140,63 +142,64 @@ __device__ __forceinline__ void unshift_axis(float (&c)[3][3][3], float v) {
 // rho G(u) - M w for the cube, telescoped so every term carries a small
 // factor: with g = e + d per axis (e = (1, 0, c_s^2), d = (0, u, u^2)),
 // rho g_a g_b g_c - e_a e_b e_c = drho g_a g_b g_c + d_a g_b g_c + e_a d_b g_c + e_a e_b d_c.
-__device__ __forceinline__ void eq_dev27(float drho, float ux, float uy, float uz, float (&q)[3][3][3]) {
-    const float gx[3] = {1.0f, ux, fmaf(ux, ux, kC)}, gy[3] = {1.0f, uy, fmaf(uy, uy, kC)},
-                gz[3] = {1.0f, uz, fmaf(uz, uz, kC)};
-    const float dx[3] = {0.0f, ux, ux * ux}, dy[3] = {0.0f, uy, uy * uy}, dz[3] = {0.0f, uz, uz * uz};
-    const float e[3] = {1.0f, 0.0f, kC};
+// Calls use(a, b, c, value) for each entry; the constant factors 0 and 1 are
+// left out by hand, the roundings are those of the full products.
+template <typename T, typename Use>
+__device__ __forceinline__ void eq_dev27(T drho, T ux, T uy, T uz, Use use) {
+    const T X = ux * ux, Y = uy * uy, Z = uz * uz;
+    const T gx[3] = {ux, ux, fmaf(ux, ux, mk_like(drho, kC))}, gy[3] = {uy, uy, fmaf(uy, uy, mk_like(drho, kC))},
+            gz[3] = {uz, uz, fmaf(uz, uz, mk_like(drho, kC))};  // (entry 0, which is 1, is not used)
+    const T dz[3] = {uz, uz, Z};                                // (entry 0, which is 0, is not used)
 #pragma unroll
-    for (int a = 0; a < 3; ++a)
+    for (int b = 0; b < 3; ++b)
 #pragma unroll
-        for (int b = 0; b < 3; ++b)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                const float gbc = gy[b] * gz[c];
-                q[a][b][c] = fmaf(drho, gx[a] * gbc, fmaf(dx[a], gbc, e[a] * fmaf(dy[b], gz[c], e[b] * dz[c])));
+        for (int c = 0; c < 3; ++c) {
+            // inner = d_b g_c + e_b d_c and gbc = g_b g_c
+            T inner, gbc;
+            if (b == 0) {
+                inner = dz[c];  // c = 0: zero, not used
+                gbc = gz[c];    // c = 0: one, not used
+            } else if (b == 1) {
+                inner = c == 0 ? uy : uy * gz[c];
+                gbc = inner;
+            } else {
+                inner = c == 0 ? Y : fmaf(Y, gz[c], kC * dz[c]);
+                gbc = c == 0 ? gy[2] : gy[2] * gz[c];
             }
+            const bool one = b == 0 && c == 0;  // gbc = 1, inner = 0
+            use(0, b, c, one ? drho : fmaf(drho, gbc, inner));
+            use(1, b, c, one ? fmaf(drho, ux, ux) : fmaf(drho, ux * gbc, ux * gbc));
+            use(2, b, c, one ? fmaf(drho, gx[2], X) : fmaf(drho, gx[2] * gbc, fmaf(X, gbc, kC * inner)));
+        }
 }
 
 // One collision on deviations h (cube by velocity code), in place; returns
-// drho of the pre-collision state (Eq. 9).
-template <bool FR = false>
-__device__ __forceinline__ float collide27(float (&h)[3][3][3], float Fx, float Fy, float Fz, const Rates27 &r) {
-    float m[3][3][3];
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int b = 0; b < 3; ++b)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) m[a][b][c] = h[a][b][c];
+// drho of the pre-collision state (Eq. 9). T: f1 (one node) or f2 (two).
+template <bool FR, typename T>
+__device__ __forceinline__ T collide27_t(T (&m)[3][3][3], T Fx, T Fy, T Fz, const Rates27 &r) {
     raw_axis<0>(m);
     raw_axis<1>(m);
     raw_axis<2>(m);
-    const float drho = m[0][0][0];
-    const float rho = 1.0f + drho;
-    const float inv = recip_of<FR>(rho);
-    const float jx = fmaf(0.5f, Fx, m[1][0][0]), jy = fmaf(0.5f, Fy, m[0][1][0]), jz = fmaf(0.5f, Fz, m[0][0][1]);
-    const float ux = jx * inv, uy = jy * inv, uz = jz * inv;
-    float e[3][3][3];
-    eq_dev27(drho, ux, uy, uz, e);
+    const T drho = m[0][0][0];
+    const T rho = 1.0f + drho;
+    const T inv = recip_of<FR>(rho);
+    const T jx = fmaf(0.5f, Fx, m[1][0][0]), jy = fmaf(0.5f, Fy, m[0][1][0]), jz = fmaf(0.5f, Fz, m[0][0][1]);
+    T ux = jx * inv, uy = jy * inv, uz = jz * inv;
     // non-equilibrium raw moments; exact values on the conserved ones
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int b = 0; b < 3; ++b)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) m[a][b][c] -= e[a][b][c];
-    const float hFx = 0.5f * Fx, hFy = 0.5f * Fy, hFz = 0.5f * Fz;
-    m[0][0][0] = 0.0f;
+    eq_dev27(drho, ux, uy, uz, [&](int a, int b, int c, T e) { m[a][b][c] = m[a][b][c] - e; });
+    const T hFx = 0.5f * Fx, hFy = 0.5f * Fy, hFz = 0.5f * Fz;
+    m[0][0][0] = mk_like(drho, 0.0f);
     m[1][0][0] = -hFx; m[0][1][0] = -hFy; m[0][0][1] = -hFz;
     // D = N(u) R
     shift_axis<0>(m, ux);
     shift_axis<1>(m, uy);
     shift_axis<2>(m, uz);
     // Eq. 5 on non-equilibrium central moments (s0 = s1 = 1)
-    m[0][0][0] = 0.0f;
+    m[0][0][0] = mk_like(drho, 0.0f);
     m[1][0][0] = hFx; m[0][1][0] = hFy; m[0][0][1] = hFz;
     m[1][1][0] *= r.om2; m[1][0][1] *= r.om2; m[0][1][1] *= r.om2;
     {
-        const float tr = r.cb * (m[2][0][0] + m[0][2][0] + m[0][0][2]);
+        const T tr = r.cb * (m[2][0][0] + m[0][2][0] + m[0][0][2]);
         m[2][0][0] = fmaf(r.om2, m[2][0][0], -tr);
         m[0][2][0] = fmaf(r.om2, m[0][2][0], -tr);
         m[0][0][2] = fmaf(r.om2, m[0][0][2], -tr);
@@ -214,33 +217,51 @@ __device__ __forceinline__ float collide27(float (&h)[3][3][3], float Fx, float 
     m[2][1][2] = fmaf(r.om5, m[2][1][2], r.c5 * Fy);
     m[2][2][1] = fmaf(r.om5, m[2][2][1], r.c5 * Fz);
     m[2][2][2] *= r.om6;
-    // R* = N(-u) D*, then Q = R* + (rho G - M w); first order exactly j + F/2
+    // R* = N(-u) D*
     unshift_axis<2>(m, uz);
     unshift_axis<1>(m, uy);
     unshift_axis<0>(m, ux);
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int b = 0; b < 3; ++b)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) m[a][b][c] += e[a][b][c];
+    // Q = R* + (rho G - M w); first order exactly j + F/2. The equilibrium is formed again from a velocity the compiler
+    // must treat as new, so that its 27 values do not stay live through the shifts.
+    T dr = drho;
+    hide(dr, ux, uy, uz);
+    eq_dev27(dr, ux, uy, uz, [&](int a, int b, int c, T e) { m[a][b][c] = m[a][b][c] + e; });
     m[0][0][0] = drho;
     m[1][0][0] = jx + hFx; m[0][1][0] = jy + hFy; m[0][0][1] = jz + hFz;
     inverse_axis<2>(m);
     inverse_axis<1>(m);
     inverse_axis<0>(m);
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-#pragma unroll
-        for (int b = 0; b < 3; ++b)
-#pragma unroll
-            for (int c = 0; c < 3; ++c) h[a][b][c] = m[a][b][c];
     return drho;
+}
+
+// One node (float: on f1, which rounds every operation on its own, so that it
+// matches the pair form bit for bit) or two (f2).
+template <bool FR = false, typename T>
+__device__ __forceinline__ T collide27(T (&h)[3][3][3], T Fx, T Fy, T Fz, const Rates27 &r) {
+    if constexpr (std::is_same<T, float>::value) {
+        f1 m[3][3][3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int b = 0; b < 3; ++b)
+#pragma unroll
+                for (int c = 0; c < 3; ++c) m[a][b][c].v = h[a][b][c];
+        const f1 drho = collide27_t<FR>(m, f1{Fx}, f1{Fy}, f1{Fz}, r);
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int b = 0; b < 3; ++b)
+#pragma unroll
+                for (int c = 0; c < 3; ++c) h[a][b][c] = m[a][b][c].v;
+        return drho.v;
+    } else {
+        return collide27_t<FR>(h, Fx, Fy, Fz, r);
+    }
 }
 
 // Deviations of the generalized local equilibrium at (rho, u).
 __device__ __forceinline__ void equilibrium_dev27(float rho, float ux, float uy, float uz, float (&h)[3][3][3]) {
-    eq_dev27(rho - 1.0f, ux, uy, uz, h);
+    eq_dev27(f1{rho - 1.0f}, f1{ux}, f1{uy}, f1{uz}, [&](int a, int b, int c, f1 e) { h[a][b][c] = e.v; });
     inverse_axis<2>(h);
     inverse_axis<1>(h);
     inverse_axis<0>(h);

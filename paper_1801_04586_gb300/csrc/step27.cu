@@ -11,9 +11,9 @@ namespace clbm {
 
 // The paper's cascaded collision on D3Q27 (Sec. II).
 struct Cascaded27 {
-    template <bool FR = false>
-    static __device__ __forceinline__ float run(float (&h)[3][3][3], float Fx, float Fy, float Fz,
-                                                const Rates27 &r) {
+    static constexpr bool kPairs = true;  // also runs on f2: the staged step pairs nodes
+    template <bool FR = false, typename T>
+    static __device__ __forceinline__ T run(T (&h)[3][3][3], T Fx, T Fy, T Fz, const Rates27 &r) {
         return collide27<FR>(h, Fx, Fy, Fz, r);
     }
 };

@@ -7,6 +7,7 @@
 namespace clbm {
 
 struct Srt27 {
+    static constexpr bool kPairs = false;  // one node at a time (float only)
     template <bool FR = false>
     static __device__ __forceinline__ float run(float (&h)[3][3][3], float Fx, float Fy, float Fz,
                                                 const Rates27 &r) {

@@ -99,6 +99,14 @@ struct TilePlan {
 // 512 threads at 64 registers spilled 60-150 bytes and measured 0.51, 384
 // threads at 80 registers 0.59, one block of 512 threads with 4 buffers 0.52).
 using TmaShape27 = TmaShape<256, 2, 2, 1024>;
+// D3Q27 in node pairs (collisions with the f2 form): a pair holds 27 pairs of
+// values and its addresses, some 160 registers, so two blocks of 192 threads
+// take pairs of a 1024-node tile. Measured at 224 x 192 x 160, FP16 / FP16-SR,
+// us a step: one node per thread in TmaShape27 193 / 254; pairs in 192 x 2
+// 173 / 182, 256 x 2 (128 registers, 60-130 bytes spilled) 211 / 215, 128 x 3
+// with 640-node tiles 188 / 201, 160 x 2 194 / 205, 256 x 1 with 4 buffers
+// 192 / 207, 384 x 1 228 / 233.
+using TmaShape27P = TmaShape<192, 2, 2, 1024, true>;
 
 // Bytes of one buffer: Q x pitch stored values, then the force on the tile's
 // nodes: for a field its three components (3 x pitch floats), for a z-profile
@@ -590,6 +598,102 @@ __device__ __forceinline__ void compute_tile_pairs(const S *src, S *dst, const G
     }
 }
 
+// The D3Q27 tile two adjacent nodes at a time, as compute_tile_pairs: 9
+// populations with e_x = 0 by 32-bit shared loads, every population's two
+// results by one pair conversion and one 32-bit store. The collision forms the
+// equilibrium twice instead of keeping its 27 values (collide27_t), so a pair
+// fits the 168 registers of two blocks of 192. Same bits as compute_tile.
+template <typename C, typename S, int FM, bool WALLS, typename SH, typename R>
+__device__ __forceinline__ void compute_tile_pairs27(const S *src, S *dst, const Geom &g, const R &r,
+                                                     const ForceArgs &F, int *flag, uint32_t key, const TilePlan &p,
+                                                     int z, int y0, const unsigned char *buf, float tfx, float tfy,
+                                                     float tfz) {
+    const S *stage = reinterpret_cast<const S *>(buf);
+    const float *fst = reinterpret_cast<const float *>(buf + (size_t)kQ27 * SH::pitch * sizeof(S));
+    constexpr int TN = SH::pitch;
+    const int rows = min(p.rows, g.ny - y0);
+    const uint32_t nx = (uint32_t)g.nx;
+    const uint32_t tile = (uint32_t)rows * nx;
+    const uint32_t base = ((uint32_t)z * (uint32_t)g.ny + (uint32_t)y0) * nx;
+    for (uint32_t n = 2u * threadIdx.x; n < tile; n += 2u * SH::threads) {
+        const uint32_t rr = __umulhi(n, p.rdiv);
+        const uint32_t x = n - rr * nx;  // even
+        const uint32_t self = base + n;   // even
+        const uint32_t sm0 = x == 0 ? n + nx - 1u : n - 1u;
+        const uint32_t sp1 = x + 2u == nx ? n + 2u - nx : n + 2u;
+        f2 h[3][3][3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int b = 0; b < 3; ++b)
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    const S *row = stage + q27_index(a, b, c) * TN;
+                    if (a == 0)
+                        h[a][b][c] = f2{
+                            Codec<S>::unpack2(*reinterpret_cast<const uint32_t *>(row + CLBM_SIDX(g, n, tile - 1u)))};
+                    else if (a == 1)  // from x - 1
+                        h[a][b][c] = mk2(Codec<S>::load_plain(row + CLBM_SIDX(g, sm0, tile)),
+                                         Codec<S>::load_plain(row + CLBM_SIDX(g, n, tile)));
+                    else              // from x + 1
+                        h[a][b][c] = mk2(Codec<S>::load_plain(row + CLBM_SIDX(g, n + 1u, tile)),
+                                         Codec<S>::load_plain(row + CLBM_SIDX(g, sp1, tile)));
+                }
+        if (WALLS) {
+            const int y = y0 + (int)rr;
+            const bool wx = g.walls & 1u, wy = g.walls & 2u, wz = g.walls & 4u;
+            const bool xl0 = wx && x == 0, xh1 = wx && x + 2u == nx;  // x wall of node n / node n + 1
+            const bool by[3] = {false, wy && y == 0, wy && y == g.ny - 1},
+                       bz[3] = {false, wz && z == 0, wz && z == g.nz - 1};
+            if (__any_sync(__activemask(), xl0 || xh1 || by[1] || by[2] || bz[1] || bz[2])) {
+#pragma unroll
+                for (int a = 0; a < 3; ++a)
+#pragma unroll
+                    for (int b = 0; b < 3; ++b)
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) {
+                            const size_t o = (size_t)q27_index(a ? 3 - a : 0, b ? 3 - b : 0, c ? 3 - c : 0) * g.stride + self;
+                            if ((a == 1 && xl0) || by[b] || bz[c])
+                                h[a][b][c].v.x = Codec<S>::load(src + CLBM_IDX(g, o));
+                            if ((a == 2 && xh1) || by[b] || bz[c])
+                                h[a][b][c].v.y = Codec<S>::load(src + CLBM_IDX(g, o + 1u));
+                        }
+            }
+        }
+        f2 fx = mk2(tfx), fy = mk2(tfy), fz = mk2(tfz);
+        if (FM == kForceField) {
+            const float2 a = *reinterpret_cast<const float2 *>(fst + n);
+            const float2 b = *reinterpret_cast<const float2 *>(fst + TN + n);
+            const float2 c = *reinterpret_cast<const float2 *>(fst + 2 * TN + n);
+            fx = mk2(a.x * F.scale, a.y * F.scale);
+            fy = mk2(b.x * F.scale, b.y * F.scale);
+            fz = mk2(c.x * F.scale, c.y * F.scale);
+        } else if (FM == kForceProfileZ) {
+            fx = mk2(fst[0] * F.scale);
+            fy = mk2(fst[1] * F.scale);
+            fz = mk2(fst[2] * F.scale);
+        }
+        const f2 drho = C::template run<true>(h, fx, fy, fz, r);
+        if (!(fabsf(drho.v.x) < 0.9f) || !(fabsf(drho.v.y) < 0.9f)) atomicOr(flag, 1);
+        const uint32_t hb = Codec<S>::kStochastic ? pair_hash(self >> 1, key) : 0u;
+        uint32_t *out = reinterpret_cast<uint32_t *>(dst + CLBM_SLOTS(g, self, (kQ27 - 1) * g.stride + 1u));
+#pragma unroll
+        for (int a = 0; a < 3; ++a)
+#pragma unroll
+            for (int b = 0; b < 3; ++b)
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    const int i = q27_index(a, b, c);
+                    uint32_t w;
+                    if constexpr (Codec<S>::kStochastic)
+                        w = Codec<S>::pair_sr(h[a][b][c].v.y, h[a][b][c].v.x, pop_bits(hb, i));
+                    else
+                        w = Codec<S>::pair_rn(h[a][b][c].v.y, h[a][b][c].v.x);
+                    out[(size_t)i * (g.stride >> 1)] = w;
+                }
+    }
+}
+
 // MODE (TileMode): the A/B pull step, on a whole lattice or on a z-slab's
 // planes z0, z0 + zs, ... (those two with the send-plane stores over its
 // first and/or last plane), or one of the two in-place kinds (src == dst:
@@ -658,7 +762,13 @@ __global__ void __launch_bounds__(SH::threads, SH::blocks)
         const bool zlo = zp == 0 && !(SLAB && (g.slab & 1u)), zhi = zp == g.nz - 1 && !(SLAB && (g.slab & 2u));
         const bool wall_tile = WALLS && ((g.walls & 1u) || ((g.walls & 4u) && (zlo || zhi)) ||
                                          ((g.walls & 2u) && (y0 == 0 || y0 + p.rows >= g.ny)));
-        if constexpr (SH::pairs) {
+        if constexpr (SH::pairs && Q == 27) {
+            const unsigned char *b = buf + s * SB;
+            if (wall_tile)
+                compute_tile_pairs27<C, S, FM, true, SH>(src, dst, g, r, F, flag, key, p, zp, y0, b, tfx, tfy, tfz);
+            else
+                compute_tile_pairs27<C, S, FM, false, SH>(src, dst, g, r, F, flag, key, p, zp, y0, b, tfx, tfy, tfz);
+        } else if constexpr (SH::pairs) {
             const unsigned char *b = buf + s * SB;
             if (wall_tile)
                 compute_tile_pairs<C, S, FM, true, SH, MODE>(src, dst, g, r, F, flag, key, p, zp, y0, b, tfx, tfy,
@@ -762,9 +872,9 @@ bool launch_step_tma(const Launch &L, const void *src, void *dst, const R &r, co
                      uint32_t key, cudaError_t &err) {
     if constexpr (Q == 27) {
         static_assert(MODE == kTilePull, "D3Q27: the A/B pull step");
-        return L.g.walls ? launch_step_tma_shape<TmaShape27, true, Q, C, S, FM, MODE>(L, src, dst, r, F, flag, key, err)
-                         : launch_step_tma_shape<TmaShape27, false, Q, C, S, FM, MODE>(L, src, dst, r, F, flag, key,
-                                                                                      err);
+        using SH = std::conditional_t<C::kPairs, TmaShape27P, TmaShape27>;
+        return L.g.walls ? launch_step_tma_shape<SH, true, Q, C, S, FM, MODE>(L, src, dst, r, F, flag, key, err)
+                         : launch_step_tma_shape<SH, false, Q, C, S, FM, MODE>(L, src, dst, r, F, flag, key, err);
     } else if constexpr (C::kPairs) {
         if constexpr (MODE == kTileAAEven)  // reads only its own slots: no wall code
             return launch_step_tma_shape<TmaShape19P, false, Q, C, S, FM, MODE>(L, src, dst, r, F, flag, key, err);
