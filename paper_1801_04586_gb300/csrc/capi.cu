@@ -383,8 +383,9 @@ int clbm_create(const clbm_params *p, void *stream, clbm_ctx **out) {
     c->gamma = 0.0;
     c->q = q;
     c->packed = q == 19 && p->variant == 2;
-    // pairs: A/B cascaded D3Q19 steps that are not staged, unless the caller chose a block of the one-node kernel
-    c->pairs = q == 19 && p->variant == 0 && p->pattern == CLBM_PATTERN_AB && p->model == CLBM_MODEL_CASCADED &&
+    // pairs: cascaded D3Q19 steps that are not staged (in place: FP32), unless the caller chose a block of the
+    // one-node kernel
+    c->pairs = q == 19 && p->variant == 0 && p->model == CLBM_MODEL_CASCADED &&
                !p->slab && p->block_x == 0 && p->block_y == 0 && step_pairs(c->g);
     // staged: A/B steps, and the cascaded D3Q19 in-place step (node pairs); they run so from staged_min_nodes on
     c->staged = p->variant == 0 &&

@@ -102,6 +102,8 @@ cudaError_t launch_step(int storage, const Launch &L, const void *src, void *dst
 bool step_pairs(const Geom &g);
 cudaError_t launch_step_pair(int storage, const Launch &L, const void *src, void *dst, const Rates &r,
                              const ForceArgs &F, int *flag, uint32_t key);
+// The in-place FP32 step in node pairs, as launch_step_aa.
+cudaError_t launch_step_aa_pair(const Launch &L, void *f, const Rates &r, const ForceArgs &F, int *flag, bool odd);
 // The cascaded step on a z-slab (Geom::slab halo faces): the planes z0,
 // z0 + zs, ... (nplanes of them) from src into dst (step.cu).
 cudaError_t launch_step_slab(int storage, const Launch &L, const void *src, void *dst, const Rates &r,

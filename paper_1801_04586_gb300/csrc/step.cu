@@ -90,6 +90,7 @@ cudaError_t launch_step_aa(int storage, const Launch &L, void *f, const Rates &r
                            uint32_t key, bool odd) {
     cudaError_t e = cudaSuccess;
     if (L.staged && launch_step_aa_staged(storage, L, f, r, F, flag, key, odd, e)) return e;
+    if (L.pairs && storage == 0) return launch_step_aa_pair(L, f, r, F, flag, odd);
     return launch_step_aa_with<Cascaded>(storage, L, f, r, F, flag, key, odd);
 }
 

@@ -46,6 +46,34 @@ static cudaError_t pair_force_t(const Launch &L, const void *src, void *dst, con
     }
 }
 
+template <int FM>
+static cudaError_t aa_pair_t(const Launch &L, void *f, const Rates &r, const ForceArgs &F, int *flag, bool odd) {
+    const Geom &g = L.g;
+    if (!odd) {
+        const uint32_t n = (uint32_t)g.nx * (uint32_t)g.ny * (uint32_t)g.nz;
+        const dim3 grid(((n + 1u) / 2u + kPairThreads - 1u) / kPairThreads);
+        return launch_overlapped(k_step_aa_pair_even<FM>, grid, dim3(kPairThreads), 0, L.stream, L.overlap, (float *)f,
+                                 g, r, F, flag, n);
+    }
+    const uint32_t npx = (uint32_t)(g.nx + 1) / 2u, rdiv = 0xffffffffu / npx + 1u;
+    const dim3 grid((npx * (uint32_t)g.ny + kPairThreads - 1u) / kPairThreads, (unsigned)g.nz);
+    auto go = [&](auto kern) {
+        return launch_overlapped(kern, grid, dim3(kPairThreads), 0, L.stream, L.overlap, (float *)f, g, r, F, flag, npx,
+                                 rdiv);
+    };
+    const bool vec = g.nx % 2 == 0;
+    if (g.walls) return vec ? go(k_step_aa_pair_odd<FM, true, true>) : go(k_step_aa_pair_odd<FM, true, false>);
+    return vec ? go(k_step_aa_pair_odd<FM, false, true>) : go(k_step_aa_pair_odd<FM, false, false>);
+}
+
+cudaError_t launch_step_aa_pair(const Launch &L, void *f, const Rates &r, const ForceArgs &F, int *flag, bool odd) {
+    switch (F.mode) {
+        case kForceUniform: return aa_pair_t<kForceUniform>(L, f, r, F, flag, odd);
+        case kForceProfileZ: return aa_pair_t<kForceProfileZ>(L, f, r, F, flag, odd);
+        default: return aa_pair_t<kForceField>(L, f, r, F, flag, odd);
+    }
+}
+
 cudaError_t launch_step_pair(int storage, const Launch &L, const void *src, void *dst, const Rates &r,
                              const ForceArgs &F, int *flag, uint32_t key) {
     switch (storage) {

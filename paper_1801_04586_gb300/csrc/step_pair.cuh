@@ -115,6 +115,134 @@ __global__ void __launch_bounds__(kPairThreads) k_step_pair(const float *src, fl
     }
 }
 
+// The in-place (AA) step with FP32 storage in node pairs (the kinds of
+// k_step_aa, step_kernels.cuh, with its bits).
+//   even kind: no node looks at a neighbour, so the pairs are 2t and 2t + 1 in
+//              the lattice's linear order, aligned whatever nx is;
+//   odd kind:  pairs of a row as k_step_pair; population i of both nodes is
+//              read from array ibar at x - e_i (from array i at a wall) and
+//              pushed to (i, x + e_i) (to array ibar at a wall): with e_x = 0
+//              both are one aligned pair, otherwise two values.
+// One node per thread, the odd kind's pushes and the idle lanes of rows that no
+// block width divides cost 12-30 % over the even kind. us a step, mean of both
+// kinds, one node / pairs: 256^3 399 / 366 (6.97 TB/s algorithmic), 200 x 180 x
+// 160 with z walls 158 / 131, 150 x 91 x 61 with a force field 21.0 / 15.7,
+// 80^3 14.3 / 10.3.
+template <int FM>
+__global__ void __launch_bounds__(kPairThreads) k_step_aa_pair_even(float *f, Geom g, Rates r, ForceArgs F,
+                                                                    int *__restrict__ flag, uint32_t n) {
+    grid_dependency_wait();
+    const uint32_t self = 2u * (blockIdx.x * kPairThreads + threadIdx.x);
+    if (self >= n) return;
+    const bool two = self + 1u < n;  // (the slot after an odd lattice's last node is padding of the array)
+    f2 h[kQ];
+#pragma unroll
+    for (int i = 0; i < kQ; ++i) h[i] = f2{ld_state2(f + (size_t)i * g.stride + CLBM_IDX(g, self))};
+    const uint32_t last = two ? self + 1u : self, plane = (uint32_t)g.nx * (uint32_t)g.ny;
+    const int za = FM == kForceProfileZ ? (int)(self / plane) : 0, zb = FM == kForceProfileZ ? (int)(last / plane) : 0;
+    f2 fx, fy, fz;
+    force_at<FM>(F, g, za, self, fx.v.x, fy.v.x, fz.v.x);
+    force_at<FM>(F, g, zb, last, fx.v.y, fy.v.y, fz.v.y);
+    const f2 drho = Cascaded::run<false>(h, fx, fy, fz, r);
+    if (!(fabsf(drho.v.x) < 0.9f) || (two && !(fabsf(drho.v.y) < 0.9f))) *flag = 1;
+#pragma unroll
+    for (int i = 0; i < kQ; ++i) {
+        float *to = f + (size_t)opposite(i) * g.stride + CLBM_IDX(g, self);
+        if (two)
+            *reinterpret_cast<float2 *>(to) = h[i].v;
+        else
+            to[0] = h[i].v.x;
+    }
+}
+
+template <int FM, bool WALLS, bool VEC>
+__global__ void __launch_bounds__(kPairThreads) k_step_aa_pair_odd(float *f, Geom g, Rates r, ForceArgs F,
+                                                                   int *__restrict__ flag, uint32_t npx,
+                                                                   uint32_t rdiv) {
+    grid_dependency_wait();
+    const uint32_t t = blockIdx.x * kPairThreads + threadIdx.x;
+    if (t >= npx * (uint32_t)g.ny) return;
+    int y = (int)__umulhi(t, rdiv), z = blockIdx.y;
+    int x = 2 * (int)(t - (uint32_t)y * npx);
+    const bool two = VEC || x + 1 < g.nx;
+    const uint32_t unx = (uint32_t)g.nx, plane = unx * (uint32_t)g.ny;
+    f2 h[kQ];
+    WallFaces wa, wb;
+    bool any = false;
+    if (WALLS) {
+        wa = wall_faces(g, x, y, z);
+        wb = wall_faces(g, two ? x + 1 : x, y, z);
+        any = wa.any() || wb.any();
+    }
+    uint32_t self;
+    {
+        const uint32_t rc = (uint32_t)y * unx, rm = (uint32_t)(y == 0 ? g.ny - 1 : y - 1) * unx,
+                       rp = (uint32_t)(y == g.ny - 1 ? 0 : y + 1) * unx;
+        const uint32_t zc = (uint32_t)z * plane, zm = (uint32_t)(z == 0 ? g.nz - 1 : z - 1) * plane,
+                       zp = (uint32_t)(z == g.nz - 1 ? 0 : z + 1) * plane;
+        const uint32_t xa = (uint32_t)x, xb = two ? xa + 1u : xa;
+        const uint32_t xam = xa == 0u ? unx - 1u : xa - 1u, xbp = xb == unx - 1u ? 0u : xb + 1u;
+        self = zc + rc + xa;
+#pragma unroll
+        for (int i = 0; i < kQ; ++i) {
+            const float *base = f + (size_t)opposite(i) * g.stride;
+            const uint32_t row =
+                (ez19(i) > 0 ? zm : (ez19(i) < 0 ? zp : zc)) + (ey19(i) > 0 ? rm : (ey19(i) < 0 ? rp : rc));
+            if (ex19(i) == 0 && VEC)
+                h[i] = f2{ld_state2(base + CLBM_IDX(g, row + xa))};
+            else if (ex19(i) == 0)
+                h[i] = mk2(ld_state(base + CLBM_IDX(g, row + xa)), ld_state(base + CLBM_IDX(g, row + xb)));
+            else if (ex19(i) > 0)
+                h[i] = mk2(ld_state(base + CLBM_IDX(g, row + xam)), ld_state(base + CLBM_IDX(g, row + (two ? xa : xam))));
+            else
+                h[i] = mk2(ld_state(base + CLBM_IDX(g, row + (two ? xb : xbp))), ld_state(base + CLBM_IDX(g, row + xbp)));
+        }
+        if (WALLS && any) {
+#pragma unroll
+            for (int i = 1; i < kQ; ++i) {
+                const float *base = f + (size_t)i * g.stride;
+                if (wa.bounces(i)) h[i].v.x = ld_state(base + CLBM_IDX(g, self));
+                if (wb.bounces(i)) h[i].v.y = ld_state(base + CLBM_IDX(g, self + (xb - xa)));
+            }
+        }
+    }
+    f2 fx, fy, fz;
+    force_at<FM>(F, g, z, self, fx.v.x, fy.v.x, fz.v.x);
+    if (FM == kForceField)
+        force_at<FM>(F, g, z, self + (two ? 1u : 0u), fx.v.y, fy.v.y, fz.v.y);
+    else
+        fx.v.y = fx.v.x, fy.v.y = fy.v.x, fz.v.y = fz.v.x;
+    const f2 drho = Cascaded::run<false>(h, fx, fy, fz, r);
+    if (!(fabsf(drho.v.x) < 0.9f) || !(fabsf(drho.v.y) < 0.9f)) *flag = 1;
+    // push targets, from coordinates the compiler must treat as new, so that the offsets above do not stay live
+    asm volatile("" : "+r"(x), "+r"(y), "+r"(z) : "f"(h[0].v.x), "f"(h[kQ - 1].v.x));
+    const uint32_t rc = (uint32_t)y * unx, rm = (uint32_t)(y == 0 ? g.ny - 1 : y - 1) * unx,
+                   rp = (uint32_t)(y == g.ny - 1 ? 0 : y + 1) * unx;
+    const uint32_t zc = (uint32_t)z * plane, zm = (uint32_t)(z == 0 ? g.nz - 1 : z - 1) * plane,
+                   zp = (uint32_t)(z == g.nz - 1 ? 0 : z + 1) * plane;
+    const uint32_t xa = (uint32_t)x, xb = two ? xa + 1u : xa;
+    const uint32_t xam = xa == 0u ? unx - 1u : xa - 1u, xbp = xb == unx - 1u ? 0u : xb + 1u;
+#pragma unroll
+    for (int i = 0; i < kQ; ++i) {
+        float *base = f + (size_t)i * g.stride;
+        const uint32_t row = (ez19(i) > 0 ? zp : (ez19(i) < 0 ? zm : zc)) + (ey19(i) > 0 ? rp : (ey19(i) < 0 ? rm : rc));
+        bool ba = false, bb = false;  // leaving through a wall: the direction that arrives from it is ibar
+        if (WALLS && any) {
+            ba = wa.bounces(opposite(i));
+            bb = wb.bounces(opposite(i));
+        }
+        if (ex19(i) == 0 && VEC && !(WALLS && any)) {
+            *reinterpret_cast<float2 *>(base + CLBM_IDX(g, row + xa)) = h[i].v;
+        } else {
+            float *back = f + (size_t)opposite(i) * g.stride + CLBM_IDX(g, self);
+            const uint32_t oa = row + (ex19(i) > 0 ? (two ? xb : xbp) : (ex19(i) < 0 ? xam : xa));
+            const uint32_t ob = row + (ex19(i) > 0 ? xbp : (ex19(i) < 0 ? xa : xb));
+            *(ba ? back : base + CLBM_IDX(g, oa)) = h[i].v.x;
+            if (two) *(bb ? back + 1 : base + CLBM_IDX(g, ob)) = h[i].v.y;
+        }
+    }
+}
+
 template <typename S>
 __device__ __forceinline__ float2 ld_state2(const S *p) {  // 16-bit formats: one word
     uint32_t w;

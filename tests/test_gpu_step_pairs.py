@@ -1,4 +1,4 @@
-"""The FP32 A/B step with two adjacent nodes per thread (csrc/step_pair.cuh),
+"""The FP32 A/B and in-place steps with two adjacent nodes per thread (csrc/step_pair.cuh),
 the default of cascaded D3Q19 lattices of 100,000 nodes or more, against the
 one-node step (variant 1): the pair rounds like the single node, so every
 population must be the same bits. Shapes: rows of even and odd length (an odd
@@ -26,17 +26,21 @@ CASES = [
     ((512, 200, 1), 4, "uniform"),   # nz = 1 between two z walls
     ((1000, 11, 10), 2, "field"),      # rows longer than a block
 ]
+# in place too: even and odd kinds, and a lattice of an odd number of nodes (the even kind's last pair is one node)
+IN_PLACE = CASES + [((75, 55, 27), 7, "field"), ((75, 55, 27), 0, "profile")]
+ALL = [(*c, "ab") for c in CASES] + [(*c, "aa") for c in IN_PLACE]
 
 
-@pytest.mark.parametrize("shape_xyz,walls,force", CASES)
-def test_pair_step_equals_one_node_step(shape_xyz, walls, force):
+@pytest.mark.parametrize("shape_xyz,walls,force,pattern", ALL)
+def test_pair_step_equals_one_node_step(shape_xyz, walls, force, pattern):
     nx, ny, nz = shape_xyz
     shape = (nz, ny, nx)
     rho = synthetic.density_perturbation(shape, 0.01, seed=601)
     u = synthetic.uniform_perturbation(shape, 0.03, seed=602)
     out = []
     for variant in (0, 1):
-        g = Lattice(nx, ny, nz, 0.02, walls=walls, s2b=1.2, s3=1.1, s4=0.9, variant=variant, device=dev())
+        g = Lattice(nx, ny, nz, 0.02, walls=walls, s2b=1.2, s3=1.1, s4=0.9, variant=variant, pattern=pattern,
+                    device=dev())
         if force == "field":
             g.set_force_field(t(synthetic.gaussian_force(shape, 1e-4, seed=603)))
         elif force == "profile":
@@ -45,7 +49,9 @@ def test_pair_step_equals_one_node_step(shape_xyz, walls, force):
             g.set_force_uniform(1e-5, -2e-5, 3e-6)
         g.init_equilibrium(t(rho), t(u))
         g.step(7)
+        first = g.populations(deviation=True)
+        g.step(1)
         g.check()
-        out.append(g.populations(deviation=True))
+        out.append((first, g.populations(deviation=True)))
         g.close()
-    assert torch.equal(out[0], out[1])
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
