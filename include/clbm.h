@@ -245,7 +245,8 @@ int clbm_set_force_decay(clbm_ctx *ctx, double gamma);
 int clbm_init_equilibrium(clbm_ctx *ctx, const float *rho_dev, const float *u_dev);
 
 /* Advance nsteps >= 0 time steps. Each step is one launch of the fused pull
- * kernel: for every node it gathers the post-collision populations of the
+ * kernel (small cascaded D3Q19 FP32 A/B lattices, below 100,000 nodes, may take
+ * two steps per launch, with the same results): for every node it gathers the post-collision populations of the
  * neighbours (Eq. 8, periodic wrap, or halfway bounce-back f_i <- f*_ibar at
  * a wall face), forms rho and u (Eq. 9), raw moments T = M f (Eq. A4),
  * central moments N(u) T (Eq. 4), relaxes them with S, T~eq and C

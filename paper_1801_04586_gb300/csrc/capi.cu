@@ -96,6 +96,8 @@ struct clbm_ctx {
     dim3 block;
     cudaStream_t cap_stream;   // private stream for graph capture (first use)
     cudaGraphExec_t graph;     // kGraphSteps steps from phase 0; null until built, dropped when the force changes
+    bool two_step;             // small FP32 lattices: pairs of steps in one launch (step_small.cu)
+    SmallPlan small;
     bool slab_pending;         // z-slab: CLBM_SLAB_FACES done, CLBM_SLAB_INTERIOR not yet
     cudaStream_t io_stream;    // clbm_run_host: host copies in plane chunks beside init / read-out (first use)
     cudaEvent_t io_ev[kIoChunks];
@@ -254,6 +256,13 @@ cudaError_t one_step(const clbm_ctx *c, const Launch &L, int cur, int64_t step) 
                       : step19(c, L, c->buf[cur], c->buf[cur ^ 1], F, key);
 }
 
+// Two time steps `step` and `step` + 1 in one launch from buffer cur into the
+// other one (contexts with two_step set).
+cudaError_t two_steps(const clbm_ctx *c, const Launch &L, int cur, int64_t step) {
+    return launch_step_small2(L, c->small, c->buf[cur], c->buf[cur ^ 1], c->rates, force_at(c, step),
+                              force_at(c, step + 1).scale, c->d_flag);
+}
+
 // Capture kGraphSteps steps starting from phase 0 (A/B: from buffer 0; AA: an
 // even step) on a private stream. Only for launches whose arguments do not
 // change from step to step: a static force and no stochastic dither key.
@@ -271,7 +280,10 @@ int ensure_graph(clbm_ctx *c) {
     cudaGraph_t g = nullptr;
     if ((e = cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal)) != cudaSuccess)
         return cuda_fail(e, "clbm_step: begin capture");
-    for (int k = 0; k < kGraphSteps && e == cudaSuccess; ++k) e = one_step(c, L, k & 1, k);
+    if (c->two_step && c->small.in_graph)  // (kGraphSteps is a multiple of 4: the buffers end in the phase they started from)
+        for (int k = 0; k < kGraphSteps / 2 && e == cudaSuccess; ++k) e = two_steps(c, L, k & 1, 2 * k);
+    else
+        for (int k = 0; k < kGraphSteps && e == cudaSuccess; ++k) e = one_step(c, L, k & 1, k);
     cudaError_t e2 = cudaStreamEndCapture(c->cap_stream, &g);
     if (e == cudaSuccess) e = e2;
     if (e == cudaSuccess) e = cudaGraphInstantiate(&c->graph, g, 0);
@@ -393,6 +405,8 @@ int clbm_create(const clbm_params *p, void *stream, clbm_ctx **out) {
     c->run_staged = c->staged && n >= staged_min_nodes(*p, q, c->pairs);
     c->aa = p->pattern == CLBM_PATTERN_AA;
     c->model = p->model;
+    c->two_step = q == 19 && p->variant == 0 && p->storage == CLBM_STORAGE_F32 && p->pattern == CLBM_PATTERN_AB &&
+                  p->model == CLBM_MODEL_CASCADED && p->block_x == 0 && p->block_y == 0 && small_plan(c->g, c->small);
     c->rates27.om2 = c->rates.om2;
     c->rates27.cb = c->rates.cb;
     c->rates27.om3 = c->rates.om3;
@@ -560,6 +574,12 @@ int clbm_step(clbm_ctx *c, int64_t nsteps) {
             if (e != cudaSuccess) return cuda_fail(e, "clbm_step: graph launch");
             c->steps_done += kGraphSteps;
         }
+    }
+    for (; c->two_step && t + 2 <= nsteps; t += 2) {
+        cudaError_t e = two_steps(c, L, c->cur, c->steps_done);
+        if (e != cudaSuccess) return cuda_fail(e, "clbm_step");
+        c->cur ^= 1;
+        c->steps_done += 2;
     }
     for (; t < nsteps; ++t) {
         int rc = advance();

@@ -104,6 +104,18 @@ cudaError_t launch_step_pair(int storage, const Launch &L, const void *src, void
                              const ForceArgs &F, int *flag, uint32_t key);
 // The in-place FP32 step in node pairs, as launch_step_aa.
 cudaError_t launch_step_aa_pair(const Launch &L, void *f, const Rates &r, const ForceArgs &F, int *flag, bool odd);
+// Two cascaded FP32 A/B steps of a small lattice in one launch (step_small.cu):
+// bricks of bx x by x bz nodes, grown by hx, hy, hz to ext = ex x ey x ez.
+struct SmallPlan {
+    int bx, by, bz, nbx, nby, nbz, hx, hy, hz;
+    int ex, ey, ext, threads;
+    int in_graph;  // pays inside a captured graph too
+    uint32_t exdiv, exydiv, bxdiv, bxydiv;  // ceil(2^32 / divisor)
+};
+bool small_plan(const Geom &g, SmallPlan &p);
+// F carries the first step's force factor, scale2 is the second step's.
+cudaError_t launch_step_small2(const Launch &L, const SmallPlan &p, const void *src, void *dst, const Rates &r,
+                               const ForceArgs &F, float scale2, int *flag);
 // The cascaded step on a z-slab (Geom::slab halo faces): the planes z0,
 // z0 + zs, ... (nplanes of them) from src into dst (step.cu).
 cudaError_t launch_step_slab(int storage, const Launch &L, const void *src, void *dst, const Rates &r,
