@@ -502,7 +502,7 @@ typedef struct clbm_batch_info {
 typedef struct clbm_batch clbm_batch;
 
 /* Create: validates every domain as clbm_create does, allocates the A/B
- * population buffers of all domains and a work list for 256-thread tiles,
+ * population buffers of all domains and a work list for a default tile size,
  * binds to `stream`. Populations start at rest (f = w). Errors: CLBM_ERR_ARG,
  * CLBM_ERR_OOM, CLBM_ERR_CUDA. */
 int clbm_batch_create(const clbm_domain *domains, int32_t ndomains, int32_t storage, void *stream,

@@ -67,12 +67,16 @@ struct DomainDesc {
     int64_t offset;        // element offset of the domain's 19 x stride block in A and in B
 };
 
-// Nodes per thread of the A/B kernel: 16-bit formats take pairs of adjacent
-// nodes (step_pair.cuh), FP32 one node. The FP32 batch runs near the DRAM rate
-// on 64 registers, which a pair does not reach (us a step of the benchmark's 64
-// domains: one node 808-818, pairs 876 at 108 registers, 1112 capped at 80);
-// the 16-bit batch is bound by instruction issue (FP16: 707-729 one node, 602
-// pairs).
+// Forms of the A/B batch, by storage and tile size T (us a step of the
+// benchmark's 64 domains, one node per thread before: FP32 808-835, FP16
+// 707-743):
+//   T up to 256 (FP32) or 128 (16-bit): pairs of adjacent nodes, one block per
+//     tile: FP32 755 (T = 64), 759 (128), 787 (256); FP16 600 (128);
+//   larger T: a grid of resident blocks that walks the tiles, one node per
+//     thread with FP32 (808 at 512; pairs 876 at 108 registers), pairs with 16
+//     bits (621 at 256, 571 at 512).
+__host__ __device__ constexpr bool one_block_per_tile(bool f32, int threads) { return threads <= (f32 ? 256 : 128); }
+// Nodes per thread of the walking kernel.
 template <typename S>
 constexpr int kBatchNodes = sizeof(S) == 2 ? 2 : 1;
 
@@ -131,6 +135,86 @@ __global__ void __launch_bounds__(512) k_batch_step(const S *A, S *__restrict__ 
             }
         }
         tile = next;
+    }
+}
+
+// The A/B batch in node pairs, one block per tile (small tiles, see
+// one_block_per_tile): no loop state and no shared domain table, so that the FP32 pair
+// keeps the 80 registers of six blocks of 128 per SM (12 bytes spilled).
+template <typename S, int MAXT>
+__global__ void __launch_bounds__(MAXT, sizeof(S) == 2 ? 5 : (MAXT == 128 ? 6 : 3))
+    k_batch_pair(const S *A, S *__restrict__ B, const DomainDesc *__restrict__ doms, const int4 *__restrict__ tiles,
+                 int *__restrict__ flag) {
+    const int4 tile = __ldg(tiles + blockIdx.x);  // (domain, pair of the row, y, z) of the tile's first pair
+    const DomainDesc *D = doms + tile.x;
+    const Geom g = D->g;
+    const float inv_npx = D->inv_npx, inv_ny = D->inv_ny;
+    const int64_t off = D->offset;
+    grid_dependency_wait();  // (the domain table and the work list stay unchanged while steps run)
+    const int npx = (g.nx + 1) >> 1;
+    const int xt = tile.y + (int)threadIdx.x;
+    const int cy = (int)(((float)xt + 0.5f) * inv_npx);
+    const int yt = tile.z + cy;
+    const int cz = (int)(((float)yt + 0.5f) * inv_ny);
+    const int x = 2 * (xt - cy * npx), y = yt - cz * g.ny, z = tile.w + cz;
+    if (z >= g.nz) return;
+    const S *src = A + off;
+    S *dst = B + off;
+    const bool even = (g.nx & 1) == 0, two = x + 1 < g.nx;
+    f2 h[kQ];
+    if constexpr (sizeof(S) == 2) {
+        const uint32_t self = even ? pair_load<S, true, true>(src, g, x, y, z, true, h)
+                                   : pair_load<S, true, false>(src, g, x, y, z, two, h);
+        const f2 drho = collide<true>(h, mk2(D->fx), mk2(D->fy), mk2(D->fz), D->r);
+        if (!(fabsf(drho.v.x) < 0.9f) || !(fabsf(drho.v.y) < 0.9f)) *flag = 1;
+        if (even)
+            pair_store<S, true>(dst, g, self, true, h, 0u);
+        else
+            pair_store<S, false>(dst, g, self, two, h, 0u);
+    } else {  // the pull of k_step_pair, rows of either parity
+        const uint32_t unx = (uint32_t)g.nx, plane = unx * (uint32_t)g.ny;
+        const uint32_t rc = (uint32_t)y * unx, rm = (uint32_t)(y == 0 ? g.ny - 1 : y - 1) * unx,
+                       rp = (uint32_t)(y == g.ny - 1 ? 0 : y + 1) * unx;
+        const uint32_t zc = (uint32_t)z * plane, zm = (uint32_t)(z == 0 ? g.nz - 1 : z - 1) * plane,
+                       zp = (uint32_t)(z == g.nz - 1 ? 0 : z + 1) * plane;
+        const uint32_t xa = (uint32_t)x, xb = two ? xa + 1u : xa;
+        const uint32_t xam = xa == 0u ? unx - 1u : xa - 1u, xbp = xb == unx - 1u ? 0u : xb + 1u;
+        const uint32_t self = zc + rc + xa;
+#pragma unroll
+        for (int i = 0; i < kQ; ++i) {
+            const float *base = src + (size_t)i * g.stride;
+            const uint32_t row =
+                (ez19(i) > 0 ? zm : (ez19(i) < 0 ? zp : zc)) + (ey19(i) > 0 ? rm : (ey19(i) < 0 ? rp : rc));
+            if (ex19(i) > 0)
+                h[i] = mk2(ld_state(base + CLBM_IDX(g, row + xam)), ld_state(base + CLBM_IDX(g, row + (two ? xa : xam))));
+            else if (ex19(i) < 0)
+                h[i] = mk2(ld_state(base + CLBM_IDX(g, row + (two ? xb : xbp))), ld_state(base + CLBM_IDX(g, row + xbp)));
+            else if (even)
+                h[i] = f2{ld_state2(base + CLBM_IDX(g, row + xa))};
+            else
+                h[i] = mk2(ld_state(base + CLBM_IDX(g, row + xa)), ld_state(base + CLBM_IDX(g, row + xb)));
+        }
+        const WallFaces wa = wall_faces(g, (int)xa, y, z), wb = wall_faces(g, (int)xb, y, z);
+        if (wa.any() || wb.any()) {
+#pragma unroll
+            for (int i = 1; i < kQ; ++i) {
+                const float *base = src + (size_t)opposite(i) * g.stride;
+                if (wa.bounces(i)) h[i].v.x = ld_state(base + CLBM_IDX(g, self));
+                if (wb.bounces(i)) h[i].v.y = ld_state(base + CLBM_IDX(g, self + (xb - xa)));
+            }
+        }
+        const f2 drho = collide<false>(h, mk2(D->fx), mk2(D->fy), mk2(D->fz), D->r);
+        if (!(fabsf(drho.v.x) < 0.9f) || !(fabsf(drho.v.y) < 0.9f)) *flag = 1;
+#pragma unroll
+        for (int i = 0; i < kQ; ++i) {
+            float *to = dst + (size_t)i * g.stride + CLBM_SLOTS(g, self, (kQ - 1) * g.stride + (xb - xa));
+            if (even) {
+                *reinterpret_cast<float2 *>(to) = h[i].v;
+            } else {
+                to[0] = h[i].v.x;
+                if (two) to[1] = h[i].v.y;
+            }
+        }
     }
 }
 
@@ -203,6 +287,14 @@ template <typename S>
 static cudaError_t batch_launch_t(const void *A, void *B, const DomainDesc *doms, int ndom, const int4 *tiles,
                                   int ntiles, int grid, dim3 block, int *flag, cudaStream_t s, bool overlap) {
     const size_t sm = ndom <= kSmemDomains ? sizeof(DomainDesc) * ndom : 0;
+    if (one_block_per_tile(sizeof(S) == 4, (int)block.x)) {
+        auto go = [&](auto kern) {
+            return launch_overlapped(kern, dim3(ntiles), block, 0, s, overlap, (const S *)A, (S *)B, doms, tiles, flag);
+        };
+        if constexpr (sizeof(S) == 4)
+            if (block.x > 128) return go(k_batch_pair<S, 256>);
+        return go(k_batch_pair<S, 128>);
+    }
     return launch_overlapped(ndom <= kSmemDomains ? k_batch_step<S, true> : k_batch_step<S, false>, grid, block, sm, s,
                              overlap, (const S *)A, (S *)B, doms, ndom, tiles, ntiles, flag);
 }
@@ -326,12 +418,13 @@ void *domain_ptr(const clbm_batch *b, int which, int d) {
 }
 
 // Build and upload the work list for T threads per block: tiles of T
-// consecutive nodes, or pairs of nodes (kBatchNodes), domain after domain.
+// consecutive nodes, or pairs of nodes, domain after domain.
 int build_tiles(clbm_batch *b, int T) {
     std::vector<int4> tiles;
     for (int d = 0; d < b->ndom; ++d) {
         const Geom &g = b->descs[d].g;
-        const bool pairs = !b->aa && b->storage != CLBM_STORAGE_F32;  // kBatchNodes
+        const bool f32 = b->storage == CLBM_STORAGE_F32;
+        const bool pairs = !b->aa && (!f32 || one_block_per_tile(f32, T));
         const int64_t row = pairs ? (g.nx + 1) / 2 : g.nx;
         const int64_t n = row * g.ny * g.nz;
         for (int64_t s0 = 0; s0 < n; s0 += T) {
@@ -361,13 +454,18 @@ int build_tiles(clbm_batch *b, int T) {
     int sms = 0, dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    b->grid = std::max(1, std::min(b->ntiles, std::max(1, sms) * batch_occupancy(b->storage, T, b->ndom)));
+    b->grid = !b->aa && one_block_per_tile(b->storage == CLBM_STORAGE_F32, T)
+                  ? b->ntiles
+                  : std::max(1, std::min(b->ntiles, std::max(1, sms) * batch_occupancy(b->storage, T, b->ndom)));
     if (b->graph) {
         cudaGraphExecDestroy(b->graph);
         b->graph = nullptr;
     }
     return CLBM_OK;
 }
+
+// The tile size a batch starts with (clbm_batch_autotune finds its own).
+int default_tile(const clbm_batch &b) { return b.aa ? 256 : (b.storage == CLBM_STORAGE_F32 ? 128 : 512); }
 
 // One step of every domain: A/B from buffer `from`; in place, the odd kind when
 // `from` is 1 (the parity of the step).
@@ -487,7 +585,7 @@ int clbm_batch_create_pattern(const clbm_domain *doms, int32_t ndomains, int32_t
                         b->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->d_flag, 0, sizeof(int), b->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->buf[0], 0, nbuf * (size_t)off * b->elem, b->stream);
-    int rc = e == cudaSuccess ? build_tiles(b, 256) : bcuda(e, "clbm_batch_create");
+    int rc = e == cudaSuccess ? build_tiles(b, default_tile(*b)) : bcuda(e, "clbm_batch_create");
     if (rc != CLBM_OK) {
         clbm_batch_destroy(b);
         return rc;
