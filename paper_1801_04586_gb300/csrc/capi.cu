@@ -177,30 +177,41 @@ Launch step_launch_of(const clbm_ctx *c) {
     return L;
 }
 
-// The smallest lattice whose 16-bit steps run staged. A staged block works
-// through tiles of 768-1024 nodes, so a small lattice leaves most SMs idle and
-// the rest with one tile's copy latency and nothing behind it. Measured (us a
-// step, staged / the form that replaces it):
+// Whether a lattice's 16-bit steps run staged. The staged blocks work through
+// tiles of up to 1024 nodes, two blocks per SM: a lattice of fewer tiles, or of
+// little more than one round of them, leaves SMs idle or waiting on one tile's
+// copy latency. Measured (us a step, staged / the form that replaces it):
 //   A/B cascaded against node pairs: FP16 48^3 4.9 / 3.0, 80^3 10.3 / 9.2,
-//     104^3 20.4 / 18.0, 128^3 34.4 / 36.9, 256^3 228 / 271; FP16-SR 48^3
-//     6.8 / 4.3, 104^3 22.4 / 19.0, 128^3 37.3 / 37.9, 256^3 251 / 278;
-//     against one node per thread (below 100,000 nodes) 32^3 6.1 / 2.2;
-//   A/B SRT and MRT against one node: 64^3 6.7 / 5.8, 96^3 17.5 / 15.7, 128^3
-//     36.4 / 36.8;
-//   in place against one node: FP16 32^3 4.9 / 2.2, 64^3 6.8 / 6.3, 80^3 11.0
-//     / 12.6; FP16-SR 64^3 7.7 / 7.5, 80^3 12.0 / 15.3;
-//   D3Q27 against one node: FP16 80^3 15.6 / 20.2, 128^3 56 / 64; FP16-SR 80^3
-//     16.2 / 24.4, 128^3 58 / 78; one tile per plane and SM below that (32^3
-//     7.2 / 2.8 and 64^3 with walls 17.4 / 10.2 in the one-node staged form).
+//     104^3 20.4 / 18.0, 112^3 23.4 / 24.8, 128^3 34.4 / 36.9, 256^3 228 / 271;
+//     FP16-SR 48^3 6.8 / 4.3, 104^3 22.4 / 19.0, 112^3 25.6 / 25.0, 128^3 37.3
+//     / 37.9, 256^3 251 / 278; below 100,000 nodes against one node per thread
+//     32^3 6.1 / 2.2;
+//   A/B SRT and MRT against one node: 64^3 6.7 / 5.8, 96^3 17.5 / 15.7, 104^3
+//     with walls 23.0 / 27.2, 112^3 24.8 / 27.7;
+//   in place and D3Q27 against one node, by the share of the rounds' tiles
+//     that are full: in place FP16 56^3 (0.56) 7.0 / 5.2, 64^3 (0.84) 6.7 /
+//     6.3, 80^3 (0.82) 10.9 / 12.6, 64 x 64 x 80 with walls (0.53) 9.7 / 8.4,
+//     104 x 64 x 56 (0.60) 10.2 / 11.2; BF16-SR 64^3 7.4 / 7.5, 72^3 (0.60)
+//     11.9 / 13.0; D3Q27 FP16 56^3 9.2 / 7.4, 64^3 9.2 / 9.1, 72^3 15.0 /
+//     16.3, 64 x 64 x 80 with walls 18.0 / 12.1, 200 x 32 x 40 (0.82) 9.3 /
+//     10.5; FP16-SR 64^3 9.5 / 10.9.
 // A context that bounds or injects the staged waits runs them at any size, as
 // do z-slabs (not measured across GPUs) and the bounds-checked build.
-int64_t staged_min_nodes(const clbm_params &p, int q, bool pairs) {
+bool staged_pays(const clbm_params &p, int q, bool pairs) {
 #ifdef CLBM_BOUNDS_CHECK
-    return 0;
+    return true;
 #endif
-    if (p.slab || p.inject || p.wait_cycles > 0) return 0;
-    if (q == 27 || p.pattern == CLBM_PATTERN_AA) return 400000;
-    return pairs || p.model != CLBM_MODEL_CASCADED ? 1500000 : 250000;
+    if (p.slab || p.inject || p.wait_cycles > 0) return true;
+    const int64_t n = (int64_t)p.nx * p.ny * p.nz;
+    const bool stochastic = p.storage == CLBM_STORAGE_F16_SR || p.storage == CLBM_STORAGE_BF16_SR;
+    if (q == 19 && p.pattern == CLBM_PATTERN_AB) {
+        if (p.model != CLBM_MODEL_CASCADED) return n >= 900000;
+        if (pairs) return n >= (stochastic ? 1500000 : 1200000);
+    }
+    if (n < 250000 || p.nx > 1024) return n >= 250000;
+    const int64_t rows = std::min<int64_t>(p.ny, 1024 / p.nx), tiles = (p.ny + rows - 1) / rows * p.nz;
+    const int64_t rounds = (tiles + 303) / 304;
+    return (double)n >= 0.58 * (double)rounds * 304 * 1024 || n >= 1000000;
 }
 
 bool rate_ok(double s) { return std::isfinite(s) && s > 0.0 && s < 2.0; }
@@ -399,10 +410,10 @@ int clbm_create(const clbm_params *p, void *stream, clbm_ctx **out) {
     // one-node kernel
     c->pairs = q == 19 && p->variant == 0 && p->model == CLBM_MODEL_CASCADED &&
                !p->slab && p->block_x == 0 && p->block_y == 0 && step_pairs(c->g);
-    // staged: A/B steps, and the cascaded D3Q19 in-place step (node pairs); they run so from staged_min_nodes on
+    // staged: A/B steps, and the cascaded D3Q19 in-place step (node pairs), where they pay
     c->staged = p->variant == 0 &&
                 (p->pattern != CLBM_PATTERN_AA || (q == 19 && p->model == CLBM_MODEL_CASCADED));
-    c->run_staged = c->staged && n >= staged_min_nodes(*p, q, c->pairs);
+    c->run_staged = c->staged && staged_pays(*p, q, c->pairs);
     c->aa = p->pattern == CLBM_PATTERN_AA;
     c->model = p->model;
     c->two_step = q == 19 && p->variant == 0 && p->storage == CLBM_STORAGE_F32 && p->pattern == CLBM_PATTERN_AB &&
