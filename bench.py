@@ -104,8 +104,8 @@ def measured_peaks():
 
 def kernel_source_digest():
     h = hashlib.sha256()
-    # the headers that define the FP32 step kernel (step.cu only instantiates it)
-    for rel in ("paper_1801_04586_gb300/csrc/step_kernels.cuh", "paper_1801_04586_gb300/csrc/d3q19.cuh",
+    # the headers that define the FP32 step kernel (step_pair.cu only instantiates it)
+    for rel in ("paper_1801_04586_gb300/csrc/step_pair.cuh", "paper_1801_04586_gb300/csrc/d3q19.cuh",
                 "paper_1801_04586_gb300/csrc/cascaded.cuh"):
         with open(os.path.join(ROOT, rel), "rb") as fh:
             h.update(fh.read())
@@ -115,7 +115,7 @@ def kernel_source_digest():
 def profiled_traffic():
     """DRAM bytes per launch of the step kernel from the committed ncu summary,
     if the kernel sources still match the digest recorded there."""
-    path = os.path.join(ROOT, "profiles", "k_step_f32_kolmogorov256.md")
+    path = os.path.join(ROOT, "profiles", "k_step_pair_f32_kolmogorov256.md")
     try:
         text = open(path).read()
     except OSError:
@@ -763,7 +763,8 @@ def run_gb300(args):
             "config": {"workload": workload,
                        "nx": nxy, "ny": nxy, "nz": gside if strong else nzl * (ws if slab else 1), "nu": NU, "F0": F0,
                        "storage": f"{args.storage} {args.pattern.upper()} "
-                                  + ("staged in shared memory" if info["staged"] else "one node per thread"),
+                                  + ("two adjacent nodes per thread" if default_case else
+                                     "staged in shared memory" if info["staged"] else "one node per thread"),
                        "block": [info["block_x"], info["block_y"]],
                        "l2": f"inputs larger than L2: {info['buffers']} population buffer(s) of "
                              f"{info['state_bytes'] / 1e9:.2f} GB vs 129 MB L2, no flush",
@@ -772,7 +773,7 @@ def run_gb300(args):
                          "frac": achieved / peak, "traffic": traffic, "peak_kind": peak_kind,
                          "frac_of_nominal": achieved / NOMINAL_HBM_GBS,
                          "algorithmic_bytes_per_launch": bytes_per_node * nodes,
-                         "kernel": "k_step<Cascaded,float,1,false>" if default_case
+                         "kernel": "k_step_pair<1,false,true>" if default_case
                          else f"step kernel, {args.model} collision, {args.storage} storage, D3Q{args.lattice}, "
                               f"{args.pattern} pattern" + (", z-slab (faces + interior launches)" if slab else "")},
             "cpu_baseline": cpu,

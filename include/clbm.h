@@ -119,8 +119,7 @@ extern "C" {
  *      (unless block_x or block_y is given); one node per thread otherwise; 1: always one node per thread,
  *      plain loads (block_x, block_y apply); 2: two nodes per thread (x and
  *      x + block_x), collided together with the FP32x2 instructions (D3Q19
- *      only; measured slower on GB300 for every storage format, kept as an
- *      option). Forms 0 and 1 give bit-identical results; form 2 the same up
+ *      only; the default form is the faster one, kept as an option). Forms 0 and 1 give bit-identical results; form 2 the same up
  *      to the rounding of fused operations.
  * lattice: 19 (or 0): D3Q19 of Appendix A (Eqs. A1-A6); 27: D3Q27 of Sec. II
  *      (velocities Eq. 1, moments Eq. 12, S Eq. 13, T~eq Eq. 15, C Eq. 16).

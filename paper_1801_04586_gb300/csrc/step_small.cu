@@ -24,12 +24,11 @@ bool small_plan(const Geom &g, SmallPlan &p) {
     if (g.slab || n >= 100000) return false;
     double best = 1e300;
     auto sizes = [](int n, int most, auto use) {  // the axis whole, or its even splits
-        int last = 0;
-        for (int k = 1; k <= n; ++k) {
-            const int s = (n + k - 1) / k;
-            if (s == last || s > most) continue;
-            last = s;
+        for (int k = (n + most - 1) / most;;) {
+            const int s = (n + k - 1) / k;  // the largest part of k even ones
             use(s, (n + s - 1) / s);
+            if (s == 1) return;
+            k = (n + s - 2) / (s - 1);  // the fewest parts that are smaller
         }
     };
     sizes(g.nx, 1024, [&](int bx, int nbx) {
