@@ -473,9 +473,9 @@ int clbm_reduce_pair_noalloc(const float *a_dev, const float *b_dev, int64_t n, 
  * A batch holds ndomains complete lattices, each with its own extents, walls,
  * rates (as clbm_params) and uniform body force, all in one storage format.
  * Each domain follows exactly the per-node update of clbm_step. The batch
- * steps all domains with one launch per time step: a grid of (SMs x resident
- * blocks) walks a work list of tiles, each `threads` consecutive nodes of one
- * domain in its linear index. The batch owns its population buffers. */
+ * steps all domains with one launch per time step over a work list of tiles,
+ * each `threads` consecutive nodes, or pairs of adjacent nodes, of one domain
+ * in its linear index. The batch owns its population buffers. */
 typedef struct clbm_domain {
     int32_t nx, ny, nz;
     uint32_t walls;

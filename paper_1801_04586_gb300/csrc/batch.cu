@@ -6,10 +6,11 @@
 // kernel (pull, Eqs. 5, 7, 8, 9 in deviation form; see d3q19.cuh). The
 // domains' populations share two A/B allocations, domain after domain, each in
 // the single-lattice layout. A host-built work list cuts every domain into
-// tiles of T consecutive nodes in its linear index (T = threads per block;
-// pairs of nodes with 16-bit storage), so every lane has a node whatever the domain's extents, a warp reads
-// contiguous memory, and only a domain's last tile is partial. A grid of
-// (SMs x resident blocks) walks the list with a stride: one launch covers all
+// tiles of T consecutive nodes, or pairs of adjacent nodes, in its linear index
+// (T = threads per block), so every lane has a node whatever the domain's
+// extents, a warp reads contiguous memory, and only a domain's last tile is
+// partial. One block takes one tile, or a grid of (SMs x resident blocks) walks
+// the list with a stride (one_block_per_tile): one launch covers all
 // domains. Steps are replayed from a captured CUDA graph.
 #include <cuda_runtime.h>
 

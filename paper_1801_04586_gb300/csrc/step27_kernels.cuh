@@ -81,7 +81,7 @@ __global__ void __launch_bounds__(256, 4) k_step27(const S *src, S *__restrict__
 // opposite slot at the node; the odd kind reads the swapped pull slots and
 // writes population (a,b,c) to the slot the opposite direction was read from.
 // A node writes exactly the slots it read; a slot is read once, by the thread
-// that later overwrites it, so loads may take the read-only path.
+// that later overwrites it, so the compiler may order the loads freely.
 template <typename C, typename S, int FM, bool WALLS, bool ODD>
 __global__ void __launch_bounds__(256) k_step27_aa(S *f, Geom g, Rates27 r, ForceArgs F, int *__restrict__ flag,
                                                    uint32_t key) {

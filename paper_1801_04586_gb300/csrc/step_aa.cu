@@ -35,7 +35,7 @@ bool launch_step_aa_staged(int storage, const Launch &L, void *f, const Rates &r
         case 2: return by_type(__nv_bfloat16{});
         case 3: return by_type(HalfSR{});
         case 4: return by_type(BF16SR{});
-        default: return false;  // FP32 stays on k_step_aa
+        default: return false;  // FP32: k_step_aa or its node pairs (step_pair.cu)
     }
 }
 

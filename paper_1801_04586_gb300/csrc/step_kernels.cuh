@@ -4,7 +4,7 @@
 // Per node (x, y, z): gather the 19 post-collision populations of the previous
 // step from the neighbours x - e_i (Eq. 8; periodic wrap or halfway
 // bounce-back), collide them and store the 19 post-collision values at the
-// node itself. Loads use the read-only path so that the +-1 x-shifted reads of
+// node itself. The +-1 x-shifted reads of
 // neighbouring threads share L1 sectors; stores are coalesced and aligned. One
 // thread per node, x fastest, so each warp touches 19 contiguous 128-byte
 // segments per direction.
@@ -80,8 +80,8 @@ __global__ void __launch_bounds__(512) k_step(const S *src, S *__restrict__ dst,
 //              (i, x + e_i), or (ibar, x) when x + e_i lies beyond a wall.
 // In both kinds a node writes exactly the slots it read, and no other node
 // touches them, so the update is race-free in place. Loads may take the
-// read-only path: a slot is read once, by the thread that later overwrites
-// it, and never after a write within the launch.
+// compiler's order (ld_state): a slot is read once, by the thread that later
+// overwrites it, and never after a write within the launch.
 template <typename C, typename S, int FM, bool WALLS, bool ODD>
 __global__ void __launch_bounds__(512, sizeof(S) == 2 ? 2 : 0) k_step_aa(S *f, Geom g, Rates r, ForceArgs F, int *__restrict__ flag,
                                                  uint32_t key) {

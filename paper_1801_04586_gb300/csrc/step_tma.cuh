@@ -10,7 +10,7 @@
 // their values from shared memory at three addresses (x - 1, x, x + 1) plus
 // constant offsets, collide and store exactly as k_step does: the results
 // are bit-identical, with a fifth fewer instructions per node. FP32 storage
-// stays on k_step, which already runs at the DRAM bound.
+// is not staged: its steps (step_pair.cuh) already run at the DRAM bound.
 //
 // Tile: `rows` consecutive x-rows (y0 .. y0 + rows - 1) of one z-plane, at
 // most a pitch of nodes (TmaShape). Under the pull map of Eq. 8, population
@@ -136,7 +136,7 @@ constexpr bool tile_fits() {
 // a row must fit a tile.
 inline bool tile_plan(const Geom &g, size_t elem, const void *src, int grid, int tn, TilePlan &p, int z0 = 0,
                       int zs = 1, int nplanes = -1) {
-    if (elem != 2) return false;  // FP32 steps stay on k_step, which already runs at the DRAM bound
+    if (elem != 2) return false;  // FP32 steps (step_pair.cuh) already run at the DRAM bound
     if (g.nx > tn || ((size_t)g.nx * elem) % 16 != 0 || ((size_t)g.stride * elem) % 16 != 0 ||
         ((uintptr_t)src & 15u) != 0)
         return false;
