@@ -856,8 +856,10 @@ bool launch_step_tma_shape(const Launch &L, const void *src, void *dst, const R 
         }
         // With walls the launches do not overlap: blocks that turn up early crowd onto the SMs whose blocks met
         // few wall tiles (512 x 128 x 128 duct, FP16-SR: 138.7 us a step overlapped, 135.4 not, 136.5 before;
-        // the periodic 256^3 box 253.2 -> 251.2 overlapped).
-        launch_overlapped(kern, grid, SH::threads, smem, L.stream, L.overlap && !WALLS, (const S *)src, (S *)dst,
+        // the periodic 256^3 box 253.2 -> 251.2 overlapped). Nor does the in-place even kind, which has no wall code
+        // but follows the odd kind's wall tiles (FP16-SR, y and z walls, mean of both kinds: 88^3 17.4 -> 16.6,
+        // 512 x 24 x 32 14.0 -> 13.1, 1024 x 12 x 30 14.4 -> 13.4).
+        launch_overlapped(kern, grid, SH::threads, smem, L.stream, L.overlap && L.g.walls == 0, (const S *)src, (S *)dst,
                           L.g, r, F, flag, key, p);
         err = cudaGetLastError();
         return true;
