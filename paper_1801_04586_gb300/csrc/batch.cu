@@ -10,8 +10,7 @@
 // (T = threads per block), so every lane has a node whatever the domain's
 // extents, a warp reads contiguous memory, and only a domain's last tile is
 // partial. One block takes one tile, or a grid of (SMs x resident blocks) walks
-// the list with a stride (one_block_per_tile): one launch covers all
-// domains. Steps are replayed from a captured CUDA graph.
+// the list with a stride (form_for): one launch covers all domains. Steps are replayed from a captured CUDA graph.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -68,38 +67,30 @@ struct DomainDesc {
     int64_t offset;        // element offset of the domain's 19 x stride block in A and in B
 };
 
-// Forms of the A/B batch, by storage and tile size T (us a step of the
-// benchmark's 64 domains, one node per thread before: FP32 808-835, FP16
-// 707-743):
-//   T up to 256 (FP32) or 128 (16-bit): pairs of adjacent nodes, one block per
-//     tile: FP32 755 (T = 64), 759 (128), 787 (256); FP16 600 (128);
-//   larger T: a grid of resident blocks that walks the tiles, one node per
-//     thread with FP32 (808 at 512; pairs 876 at 108 registers), pairs with 16
-//     bits (621 at 256, 571 at 512).
-__host__ __device__ constexpr bool one_block_per_tile(bool f32, int threads) { return threads <= (f32 ? 256 : 128); }
-// Nodes per thread of the walking kernel.
-template <typename S>
-constexpr int kBatchNodes = sizeof(S) == 2 ? 2 : 1;
+// Blocks of 128 threads of the node-pair kernel that an SM holds (its launch bounds).
+__host__ __device__ constexpr int pair_blocks(bool f32) { return f32 ? 6 : 5; }
 
 // SMEM: the domain table is staged in shared memory once per launch (the
 // usual case); otherwise it is read through the read-only cache. The next
 // tile's entry is fetched while the current tile is processed. A tile is
 // blockDim.x consecutive nodes of the domain, or pairs of adjacent nodes in
 // the order of rows of (nx + 1) / 2 pairs, one per thread.
-template <typename S, bool SMEM>
+template <typename S, int NODES, bool SMEM>
 __global__ void __launch_bounds__(512) k_batch_step(const S *A, S *__restrict__ B,
                                                     const DomainDesc *__restrict__ doms, int ndom,
                                                     const int4 *__restrict__ tiles, int ntiles,
                                                     int *__restrict__ flag) {
     extern __shared__ DomainDesc sdom[];
+    int t = blockIdx.x;
+    if (t >= ntiles) return;
+    // the domain table and the work list stay unchanged while steps run; the first tile's entry is on its way while
+    // the table is staged
+    int4 tile = __ldg(tiles + t);  // (domain, x or pair of the row, y, z) of the tile's first node or pair
     if (SMEM) {
         for (int i = threadIdx.x; i < ndom; i += blockDim.x) sdom[i] = doms[i];
         __syncthreads();
     }
-    grid_dependency_wait();  // (the domain table and the work list stay unchanged while steps run)
-    int t = blockIdx.x;
-    if (t >= ntiles) return;
-    int4 tile = __ldg(tiles + t);  // (domain, x or pair of the row, y, z) of the tile's first node or pair
+    grid_dependency_wait();
     for (; t < ntiles; t += gridDim.x) {
         const int tn = t + gridDim.x;
         const int4 next = tn < ntiles ? __ldg(tiles + tn) : tile;
@@ -107,16 +98,16 @@ __global__ void __launch_bounds__(512) k_batch_step(const S *A, S *__restrict__ 
         const Geom g = D->g;
         // entry tile_start + threadIdx.x: carry x into y and y into z. The
         // quotients are below 2^17, so floor((v + 0.5) * (1/n)) in FP32 is exact.
-        const int row = kBatchNodes<S> == 2 ? (g.nx + 1) >> 1 : g.nx;
+        const int row = NODES == 2 ? (g.nx + 1) >> 1 : g.nx;
         const int xt = tile.y + (int)threadIdx.x;
-        const int cy = (int)(((float)xt + 0.5f) * (kBatchNodes<S> == 2 ? D->inv_npx : D->inv_nx));
+        const int cy = (int)(((float)xt + 0.5f) * (NODES == 2 ? D->inv_npx : D->inv_nx));
         const int yt = tile.z + cy;
         const int cz = (int)(((float)yt + 0.5f) * D->inv_ny);
-        const int x = kBatchNodes<S> * (xt - cy * row), y = yt - cz * g.ny, z = tile.w + cz;
+        const int x = NODES * (xt - cy * row), y = yt - cz * g.ny, z = tile.w + cz;
         if (z < g.nz) {
             const S *src = A + D->offset;
             S *dst = B + D->offset;
-            if constexpr (kBatchNodes<S> == 2) {
+            if constexpr (NODES == 2) {
                 const bool even = (g.nx & 1) == 0, two = x + 1 < g.nx;
                 f2 h[kQ];
                 const uint32_t self = even ? pair_load<S, true, true>(src, g, x, y, z, true, h)
@@ -130,7 +121,7 @@ __global__ void __launch_bounds__(512) k_batch_step(const S *A, S *__restrict__ 
             } else {
                 float h[kQ];
                 const uint32_t self = pull_load<S, true>(src, g, x, y, z, h);
-                const float drho = collide<false>(h, D->fx, D->fy, D->fz, D->r);
+                const float drho = collide<sizeof(S) == 2>(h, D->fx, D->fy, D->fz, D->r);
                 if (!(fabsf(drho) < 0.9f)) *flag = 1;
                 store_node<S>(dst + self, g.stride, h, self, 0u);
             }
@@ -140,10 +131,10 @@ __global__ void __launch_bounds__(512) k_batch_step(const S *A, S *__restrict__ 
 }
 
 // The A/B batch in node pairs, one block per tile (small tiles, see
-// one_block_per_tile): no loop state and no shared domain table, so that the FP32 pair
+// form_for): no loop state and no shared domain table, so that the FP32 pair
 // keeps the 80 registers of six blocks of 128 per SM (12 bytes spilled).
 template <typename S, int MAXT>
-__global__ void __launch_bounds__(MAXT, sizeof(S) == 2 ? 5 : (MAXT == 128 ? 6 : 3))
+__global__ void __launch_bounds__(MAXT, pair_blocks(sizeof(S) == 4) * 128 / MAXT)
     k_batch_pair(const S *A, S *__restrict__ B, const DomainDesc *__restrict__ doms, const int4 *__restrict__ tiles,
                  int *__restrict__ flag) {
     const int4 tile = __ldg(tiles + blockIdx.x);  // (domain, pair of the row, y, z) of the tile's first pair
@@ -233,14 +224,16 @@ __global__ void __launch_bounds__(512, ODD || sizeof(S) == 2 ? 0 : 2) k_batch_st
                                                        const int4 *__restrict__ tiles, int ntiles,
                                                        int *__restrict__ flag) {
     extern __shared__ DomainDesc sdom[];
+    int t = blockIdx.x;
+    if (t >= ntiles) return;
+    // the domain table and the work list stay unchanged while steps run; the first tile's entry is on its way while
+    // the table is staged
+    int4 tile = __ldg(tiles + t);
     if (SMEM) {
         for (int i = threadIdx.x; i < ndom; i += blockDim.x) sdom[i] = doms[i];
         __syncthreads();
     }
-    grid_dependency_wait();  // (the domain table and the work list stay unchanged while steps run)
-    int t = blockIdx.x;
-    if (t >= ntiles) return;
-    int4 tile = __ldg(tiles + t);
+    grid_dependency_wait();
     for (; t < ntiles; t += gridDim.x) {
         const int tn = t + gridDim.x;
         const int4 next = tn < ntiles ? __ldg(tiles + tn) : tile;
@@ -284,76 +277,78 @@ __global__ void __launch_bounds__(512, ODD || sizeof(S) == 2 ? 0 : 2) k_batch_st
 
 constexpr int kSmemDomains = 512;  // domain tables up to this size are staged in shared memory
 
+// The kernel of one step: how a batch's work list is cut and walked.
+struct BatchForm {
+    int threads = 0;
+    bool pairs = false;     // A/B: a thread takes two adjacent nodes instead of one
+    bool per_tile = false;  // ... and a block one tile (k_batch_pair); otherwise resident blocks walk the tiles
+};
+
+// The step kernel of a form (A/B; in place, of one kind) through `use`.
+template <typename S, typename Use>
+static auto with_kernel(const BatchForm &f, int ndom, Use use) {
+    const bool sm = ndom <= kSmemDomains;
+    if constexpr (sizeof(S) == 2)  // (FP32 pairs take one block per tile)
+        if (f.pairs) return use(sm ? k_batch_step<S, 2, true> : k_batch_step<S, 2, false>);
+    return use(sm ? k_batch_step<S, 1, true> : k_batch_step<S, 1, false>);
+}
+template <typename S, typename Use>
+static auto with_kernel_aa(bool odd, int ndom, Use use) {
+    const bool sm = ndom <= kSmemDomains;
+    if (odd) return use(sm ? k_batch_step_aa<S, true, true> : k_batch_step_aa<S, false, true>);
+    return use(sm ? k_batch_step_aa<S, true, false> : k_batch_step_aa<S, false, false>);
+}
+
+static size_t table_bytes(int ndom) { return ndom <= kSmemDomains ? sizeof(DomainDesc) * ndom : 0; }
+
 template <typename S>
-static cudaError_t batch_launch_t(const void *A, void *B, const DomainDesc *doms, int ndom, const int4 *tiles,
-                                  int ntiles, int grid, dim3 block, int *flag, cudaStream_t s, bool overlap) {
-    const size_t sm = ndom <= kSmemDomains ? sizeof(DomainDesc) * ndom : 0;
-    if (one_block_per_tile(sizeof(S) == 4, (int)block.x)) {
+static cudaError_t batch_launch_t(const BatchForm &f, const void *A, void *B, const DomainDesc *doms, int ndom,
+                                  const int4 *tiles, int ntiles, int grid, int *flag, cudaStream_t s, bool overlap) {
+    const dim3 block(f.threads);
+    if (f.per_tile) {
         auto go = [&](auto kern) {
             return launch_overlapped(kern, dim3(ntiles), block, 0, s, overlap, (const S *)A, (S *)B, doms, tiles, flag);
         };
         if constexpr (sizeof(S) == 4)
-            if (block.x > 128) return go(k_batch_pair<S, 256>);
+            if (f.threads > 128) return go(k_batch_pair<S, 256>);
         return go(k_batch_pair<S, 128>);
     }
-    return launch_overlapped(ndom <= kSmemDomains ? k_batch_step<S, true> : k_batch_step<S, false>, grid, block, sm, s,
-                             overlap, (const S *)A, (S *)B, doms, ndom, tiles, ntiles, flag);
+    return with_kernel<S>(f, ndom, [&](auto kern) {
+        return launch_overlapped(kern, dim3(grid), block, table_bytes(ndom), s, overlap, (const S *)A, (S *)B, doms,
+                                 ndom, tiles, ntiles, flag);
+    });
 }
 
 template <typename S>
-static cudaError_t batch_launch_aa_t(void *A, const DomainDesc *doms, int ndom, const int4 *tiles, int ntiles,
-                                     int grid, dim3 block, int *flag, cudaStream_t s, bool overlap,
-                                   bool odd) {
-    const size_t sm = ndom <= kSmemDomains ? sizeof(DomainDesc) * ndom : 0;
-    if (ndom <= kSmemDomains) {
-        if (odd) launch_overlapped(k_batch_step_aa<S, true, true>, grid, block, sm, s, overlap, (S *)A, doms, ndom,
-                                   tiles, ntiles, flag);
-        else launch_overlapped(k_batch_step_aa<S, true, false>, grid, block, sm, s, overlap, (S *)A, doms, ndom,
-                               tiles, ntiles, flag);
-    } else {
-        if (odd) launch_overlapped(k_batch_step_aa<S, false, true>, grid, block, 0, s, overlap, (S *)A, doms, ndom,
-                                   tiles, ntiles, flag);
-        else launch_overlapped(k_batch_step_aa<S, false, false>, grid, block, 0, s, overlap, (S *)A, doms, ndom,
-                               tiles, ntiles, flag);
-    }
-    return cudaGetLastError();
+static cudaError_t batch_launch_aa_t(const BatchForm &f, void *A, const DomainDesc *doms, int ndom, const int4 *tiles,
+                                     int ntiles, int grid, int *flag, cudaStream_t s, bool overlap, bool odd) {
+    return with_kernel_aa<S>(odd, ndom, [&](auto kern) {
+        return launch_overlapped(kern, dim3(grid), dim3(f.threads), table_bytes(ndom), s, overlap, (S *)A, doms, ndom,
+                                 tiles, ntiles, flag);
+    });
 }
 
-static cudaError_t batch_launch_aa(int storage, void *A, const DomainDesc *doms, int ndom, const int4 *tiles,
-                                   int ntiles, int grid, dim3 block, int *flag, cudaStream_t s, bool overlap,
-                                   bool odd) {
+template <typename Use>
+static auto with_storage(int storage, Use use) {
     switch (storage) {
-        case 0: return batch_launch_aa_t<float>(A, doms, ndom, tiles, ntiles, grid, block, flag, s, overlap, odd);
-        case 1: return batch_launch_aa_t<__half>(A, doms, ndom, tiles, ntiles, grid, block, flag, s, overlap, odd);
-        default: return batch_launch_aa_t<__nv_bfloat16>(A, doms, ndom, tiles, ntiles, grid, block, flag, s, overlap, odd);
+        case 0: return use(float{});
+        case 1: return use(__half{});
+        default: return use(__nv_bfloat16{});
     }
 }
 
-static cudaError_t batch_launch(int storage, const void *A, void *B, const DomainDesc *doms, int ndom,
-                                const int4 *tiles, int ntiles, int grid, dim3 block, int *flag, cudaStream_t s,
-                                bool overlap) {
-    switch (storage) {
-        case 0: return batch_launch_t<float>(A, B, doms, ndom, tiles, ntiles, grid, block, flag, s, overlap);
-        case 1: return batch_launch_t<__half>(A, B, doms, ndom, tiles, ntiles, grid, block, flag, s, overlap);
-        default: return batch_launch_t<__nv_bfloat16>(A, B, doms, ndom, tiles, ntiles, grid, block, flag, s, overlap);
-    }
-}
-
-template <typename S>
-static int occupancy_t(int threads, int ndom) {
-    int per_sm = 0;
-    const size_t sm = ndom <= kSmemDomains ? sizeof(DomainDesc) * ndom : 0;
-    const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &per_sm, ndom <= kSmemDomains ? k_batch_step<S, true> : k_batch_step<S, false>, threads, sm);
-    return (e == cudaSuccess && per_sm > 0) ? per_sm : 1;
-}
-
-static int batch_occupancy(int storage, int threads, int ndom) {
-    switch (storage) {
-        case 0: return occupancy_t<float>(threads, ndom);
-        case 1: return occupancy_t<__half>(threads, ndom);
-        default: return occupancy_t<__nv_bfloat16>(threads, ndom);
-    }
+// Resident blocks per SM of the kernel that walks the tiles (in place: of the kind `odd`).
+static int resident_blocks(int storage, const BatchForm &f, bool aa, bool odd, int ndom) {
+    auto ask = [&](auto kern) {
+        int per_sm = 0;
+        const cudaError_t e =
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, f.threads, table_bytes(ndom));
+        return e == cudaSuccess && per_sm > 0 ? per_sm : 1;
+    };
+    return with_storage(storage, [&](auto s) {
+        using S = decltype(s);
+        return aa ? with_kernel_aa<S>(odd, ndom, ask) : with_kernel<S>(f, ndom, ask);
+    });
 }
 
 }  // namespace clbm
@@ -370,12 +365,14 @@ struct clbm_batch {
     cudaStream_t stream, capture_stream;
     DomainDesc *d_descs;
     int4 *d_tiles;
-    int ntiles, tiles_cap, grid;
-    dim3 block;
+    int ntiles, tiles_cap;
+    BatchForm form;
+    int grid[2];  // of a step; in place: of the even and of the odd kind
     int *d_flag;
     cudaGraphExec_t graph;
     int graph_steps;
     int64_t steps_done;
+    int sms;  // of the device
     bool aa;  // in-place pattern: one buffer (buf[1] == buf[0]), step kind by the parity of steps_done
 };
 
@@ -418,15 +415,31 @@ void *domain_ptr(const clbm_batch *b, int which, int d) {
     return (char *)b->buf[which] + (size_t)b->descs[d].offset * b->elem;
 }
 
+// The form of tiles of T threads (us a step of the benchmark's 64 domains, one
+// node per thread before: FP32 808-835, FP16 707-743):
+//   A/B, T up to 256 (FP32) or 128 (16-bit): pairs of adjacent nodes, one block
+//     per tile: FP32 755 (T = 64), 759 (128), 787 (256); FP16 600 (128);
+//   larger T: a grid of resident blocks that walks the tiles, one node per
+//     thread with FP32 (808 at 512; pairs 876 at 108 registers), pairs with 16
+//     bits (621 at 256, 571 at 512).
+BatchForm form_for(const clbm_batch &b, int T) {
+    BatchForm f;
+    f.threads = T;
+    const bool f32 = b.storage == CLBM_STORAGE_F32;
+    if (b.aa) return f;
+    f.per_tile = T <= (f32 ? 256 : 128);
+    f.pairs = f.per_tile || !f32;
+    return f;
+}
+
 // Build and upload the work list for T threads per block: tiles of T
 // consecutive nodes, or pairs of nodes, domain after domain.
 int build_tiles(clbm_batch *b, int T) {
+    const BatchForm form = form_for(*b, T);
     std::vector<int4> tiles;
     for (int d = 0; d < b->ndom; ++d) {
         const Geom &g = b->descs[d].g;
-        const bool f32 = b->storage == CLBM_STORAGE_F32;
-        const bool pairs = !b->aa && (!f32 || one_block_per_tile(f32, T));
-        const int64_t row = pairs ? (g.nx + 1) / 2 : g.nx;
+        const int64_t row = form.pairs ? (g.nx + 1) / 2 : g.nx;
         const int64_t n = row * g.ny * g.nz;
         for (int64_t s0 = 0; s0 < n; s0 += T) {
             const int x = (int)(s0 % row);
@@ -451,13 +464,11 @@ int build_tiles(clbm_batch *b, int T) {
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return bcuda(e, "clbm_batch: work list upload");
     b->ntiles = (int)tiles.size();
-    b->block = dim3(T, 1, 1);
-    int sms = 0, dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    b->grid = !b->aa && one_block_per_tile(b->storage == CLBM_STORAGE_F32, T)
-                  ? b->ntiles
-                  : std::max(1, std::min(b->ntiles, std::max(1, sms) * batch_occupancy(b->storage, T, b->ndom)));
+    b->form = form;
+    for (int odd = 0; odd < 2; ++odd)
+        b->grid[odd] = form.per_tile
+                           ? b->ntiles
+                           : std::min(b->ntiles, b->sms * resident_blocks(b->storage, form, b->aa, odd, b->ndom));
     if (b->graph) {
         cudaGraphExecDestroy(b->graph);
         b->graph = nullptr;
@@ -465,18 +476,28 @@ int build_tiles(clbm_batch *b, int T) {
     return CLBM_OK;
 }
 
-// The tile size a batch starts with (clbm_batch_autotune finds its own).
-int default_tile(const clbm_batch &b) { return b.aa ? 256 : (b.storage == CLBM_STORAGE_F32 ? 128 : 512); }
+// The tile size a batch starts with (clbm_batch_autotune finds its own). In
+// place, us a step: 128; 16-bit batches 512 from 700,000 nodes on and 256 from
+// 3 M on, where the populations no longer fit the L2: FP16 128 / 256 / 512: 0.5 M
+// nodes 14.7 / 15.2 / 15.3, 1.7 M 45.1 / 43.9 / 43.6, 4.5 M 126.7 / 127.3 / 130.4,
+// 36 M 981 / 972 / 981 (FP32 36 M 1036 / 1063 / 1151).
+int default_tile(const clbm_batch &b) {
+    const bool f32 = b.storage == CLBM_STORAGE_F32;
+    if (b.aa) return f32 || b.total_nodes < 700000 ? 128 : (b.total_nodes < 3000000 ? 512 : 256);
+    return f32 ? 128 : 512;
+}
 
 // One step of every domain: A/B from buffer `from`; in place, the odd kind when
 // `from` is 1 (the parity of the step).
 cudaError_t launch_all(clbm_batch *b, cudaStream_t s, int from) {
     const bool overlap = s != b->capture_stream;
-    if (b->aa)
-        return batch_launch_aa(b->storage, b->buf[0], b->d_descs, b->ndom, b->d_tiles, b->ntiles, b->grid, b->block,
-                               b->d_flag, s, overlap, from == 1);
-    return batch_launch(b->storage, b->buf[from], b->buf[from ^ 1], b->d_descs, b->ndom, b->d_tiles, b->ntiles,
-                        b->grid, b->block, b->d_flag, s, overlap);
+    return with_storage(b->storage, [&](auto v) {
+        using S = decltype(v);
+        return b->aa ? batch_launch_aa_t<S>(b->form, b->buf[0], b->d_descs, b->ndom, b->d_tiles, b->ntiles,
+                                            b->grid[from], b->d_flag, s, overlap, from == 1)
+                     : batch_launch_t<S>(b->form, b->buf[from], b->buf[from ^ 1], b->d_descs, b->ndom, b->d_tiles,
+                                         b->ntiles, b->grid[0], b->d_flag, s, overlap);
+    });
 }
 
 // Capture graph_steps steps starting from buffer 0 (in place: from an even
@@ -559,6 +580,12 @@ int clbm_batch_create_pattern(const clbm_domain *doms, int32_t ndomains, int32_t
         b->host.push_back(p);
     }
     b->total_nodes = nodes;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || b->sms < 1) {
+        cudaGetLastError();
+        b->sms = 1;
+    }
     b->total_elems = off;
     const size_t nbuf = b->aa ? 1 : 2;
     cudaError_t e = cudaMalloc(&b->buf[0], nbuf * (size_t)off * b->elem);
@@ -613,8 +640,8 @@ int clbm_batch_get_info(const clbm_batch *b, clbm_batch_info *info) {
     info->total_nodes = b->total_nodes;
     info->state_bytes = (int64_t)b->total_elems * (int64_t)b->elem;
     info->ntiles = b->ntiles;
-    info->grid = b->grid;
-    info->threads = (int32_t)b->block.x;
+    info->grid = b->grid[0];
+    info->threads = b->form.threads;
     info->graph_steps = b->graph_steps;
     info->steps_done = b->steps_done;
     info->pattern = b->aa ? CLBM_PATTERN_AA : CLBM_PATTERN_AB;
