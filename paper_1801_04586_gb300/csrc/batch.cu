@@ -415,18 +415,23 @@ void *domain_ptr(const clbm_batch *b, int which, int d) {
     return (char *)b->buf[which] + (size_t)b->descs[d].offset * b->elem;
 }
 
-// The form of tiles of T threads (us a step of the benchmark's 64 domains, one
-// node per thread before: FP32 808-835, FP16 707-743):
-//   A/B, T up to 256 (FP32) or 128 (16-bit): pairs of adjacent nodes, one block
-//     per tile: FP32 755 (T = 64), 759 (128), 787 (256); FP16 600 (128);
-//   larger T: a grid of resident blocks that walks the tiles, one node per
-//     thread with FP32 (808 at 512; pairs 876 at 108 registers), pairs with 16
-//     bits (621 at 256, 571 at 512).
+// The form a batch of `nodes` nodes steps in with tiles of T threads, us a step of batches of channels and ducts:
+// A/B, by size (nodes): below 1.2 rounds of resident pair blocks (FP32 280,000,
+//   16-bit 233,000) one node per thread: half as many warps of pairs leave
+//   schedulers idle (T = 128, one node / pairs: FP16 45k 2.97 / 3.49, 94k 4.14
+//   / 4.75, 234k 6.94 / 6.95, 352k 9.76 / 9.00; FP32 94k 4.24 / 4.64, 234k 6.70
+//   / 7.25, 352k 9.45 / 8.92);
+// above that by T:
+//   up to 256 (FP32) or 128 (16-bit): pairs, one block per tile: FP32 897 (T =
+//     128) and 929 (256) on 39 M nodes, FP16 708 (128);
+//   larger: resident blocks walk the tiles, one node per thread with FP32 (976
+//     at 512; a walking pair takes 108 registers), pairs with 16 bits (726 at
+//     256, 667 at 512).
 BatchForm form_for(const clbm_batch &b, int T) {
     BatchForm f;
     f.threads = T;
     const bool f32 = b.storage == CLBM_STORAGE_F32;
-    if (b.aa) return f;
+    if (b.aa || (double)b.total_nodes < 1.2 * b.sms * pair_blocks(f32) * 256) return f;
     f.per_tile = T <= (f32 ? 256 : 128);
     f.pairs = f.per_tile || !f32;
     return f;
@@ -476,15 +481,19 @@ int build_tiles(clbm_batch *b, int T) {
     return CLBM_OK;
 }
 
-// The tile size a batch starts with (clbm_batch_autotune finds its own). In
-// place, us a step: 128; 16-bit batches 512 from 700,000 nodes on and 256 from
-// 3 M on, where the populations no longer fit the L2: FP16 128 / 256 / 512: 0.5 M
-// nodes 14.7 / 15.2 / 15.3, 1.7 M 45.1 / 43.9 / 43.6, 4.5 M 126.7 / 127.3 / 130.4,
-// 36 M 981 / 972 / 981 (FP32 36 M 1036 / 1063 / 1151).
+// The tile size a batch starts with (clbm_batch_autotune finds its own), us a step:
+// A/B: 128; 512 for 16-bit batches of 30 rounds of resident 512-thread blocks or
+//   more (one block per SM, 1024-node tiles: 4.7 M nodes), whose last round no
+//   longer counts: FP16 128 / 512: 0.5 M nodes 12.0 / 15.0, 2.2 M 46.1 / 47.1,
+//   4.5 M 88.7 / 88.5, 36 M 657 / 617.
+// In place: 128; 16-bit batches 512 from 700,000 nodes on and 256 from 3 M on,
+//   where the populations no longer fit the L2: FP16 128 / 256 / 512: 0.5 M
+//   14.7 / 15.2 / 15.3, 1.7 M 45.1 / 43.9 / 43.6, 4.5 M 126.7 / 127.3 / 130.4,
+//   36 M 981 / 972 / 981 (FP32 36 M 1036 / 1063 / 1151).
 int default_tile(const clbm_batch &b) {
-    const bool f32 = b.storage == CLBM_STORAGE_F32;
-    if (b.aa) return f32 || b.total_nodes < 700000 ? 128 : (b.total_nodes < 3000000 ? 512 : 256);
-    return f32 ? 128 : 512;
+    if (b.storage == CLBM_STORAGE_F32) return 128;
+    if (b.aa) return b.total_nodes < 700000 ? 128 : (b.total_nodes < 3000000 ? 512 : 256);
+    return b.total_nodes < (int64_t)30 * b.sms * 1024 ? 128 : 512;
 }
 
 // One step of every domain: A/B from buffer `from`; in place, the odd kind when
