@@ -82,9 +82,20 @@ __global__ void __launch_bounds__(256, 4) k_step27(const S *src, S *__restrict__
 // writes population (a,b,c) to the slot the opposite direction was read from.
 // A node writes exactly the slots it read; a slot is read once, by the thread
 // that later overwrites it, so the compiler may order the loads freely.
+// Blocks of 256 that the in-place kernel's registers are held to (0: the
+// compiler's choice). The cascaded FP32 even kind takes 93 registers by itself
+// (20 warps per SM), 80 in 24 warps when held to three blocks; a force field
+// then spills more than that gains, and the odd kind's 80 registers come out
+// faster only under a uniform force without walls. us a step, mean of both
+// kinds, free / held: 224 x 192 x 160 uniform 277.6 / 266.8, with walls 278.4 /
+// 275.0 (odd kind held too: 284.3), z profile 269.3 / 265.5, force field 274.5
+// / 296.6 (left free); 96 x 256 x 200 uniform 198.0 / 191.3.
 template <typename C, typename S, int FM, bool WALLS, bool ODD>
-__global__ void __launch_bounds__(256) k_step27_aa(S *f, Geom g, Rates27 r, ForceArgs F, int *__restrict__ flag,
-                                                   uint32_t key) {
+constexpr int kAaBlocks = C::kPairs && sizeof(S) == 4 && (ODD ? FM == kForceUniform && !WALLS : FM != kForceField) ? 3 : 0;
+
+template <typename C, typename S, int FM, bool WALLS, bool ODD>
+__global__ void __launch_bounds__(256, kAaBlocks<C, S, FM, WALLS, ODD>)
+    k_step27_aa(S *f, Geom g, Rates27 r, ForceArgs F, int *__restrict__ flag, uint32_t key) {
     grid_dependency_wait();
     int x, y, z;
     if (!node27(g, x, y, z)) return;
