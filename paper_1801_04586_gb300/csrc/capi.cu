@@ -214,6 +214,16 @@ bool staged_pays(const clbm_params &p, int q, bool pairs) {
     return (double)n >= 0.58 * (double)rounds * 304 * 1024 || n >= 1000000;
 }
 
+// SMs of the current device (1 if that cannot be asked: the allocations that follow then report the error).
+int device_sms() {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess &&
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && sms > 0)
+        return sms;
+    cudaGetLastError();
+    return 1;
+}
+
 bool rate_ok(double s) { return std::isfinite(s) && s > 0.0 && s < 2.0; }
 
 // One D3Q19 step of the context's collision model and pattern.
@@ -420,7 +430,8 @@ int clbm_create(const clbm_params *p, void *stream, clbm_ctx **out) {
     c->aa = p->pattern == CLBM_PATTERN_AA;
     c->model = p->model;
     c->two_step = q == 19 && p->variant == 0 && p->storage == CLBM_STORAGE_F32 && p->pattern == CLBM_PATTERN_AB &&
-                  p->model == CLBM_MODEL_CASCADED && p->block_x == 0 && p->block_y == 0 && small_plan(c->g, c->small);
+                  p->model == CLBM_MODEL_CASCADED && p->block_x == 0 && p->block_y == 0 &&
+                  small_plan(c->g, device_sms(), c->small);
     c->rates27.om2 = c->rates.om2;
     c->rates27.cb = c->rates.cb;
     c->rates27.om3 = c->rates.om3;

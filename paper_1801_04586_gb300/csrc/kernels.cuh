@@ -112,7 +112,7 @@ struct SmallPlan {
     int in_graph;  // pays inside a captured graph too
     uint32_t exdiv, exydiv, bxdiv, bxydiv;  // ceil(2^32 / divisor)
 };
-bool small_plan(const Geom &g, SmallPlan &p);
+bool small_plan(const Geom &g, int sms, SmallPlan &p);  // sms: SMs of the device
 // F carries the first step's force factor, scale2 is the second step's.
 cudaError_t launch_step_small2(const Launch &L, const SmallPlan &p, const void *src, void *dst, const Rates &r,
                                const ForceArgs &F, float scale2, int *flag);

@@ -10,7 +10,7 @@ namespace clbm {
 // The brick that minimises a model of the launch, in cycles: 2100 of latency
 // and 190 per warp and stage on the SM that has most of them, fitted to
 // measured launches (8^3 to 128 x 128 x 5) to some 8 %. Only plans whose blocks
-// are all resident at once are taken: 46^3 (two rounds of 800-thread blocks)
+// are all resident at once (on the sms SMs of the device) are taken: 46^3 (two rounds of 800-thread blocks)
 // measured 5.95 us a step against 4.13 one step per launch. A single step, in
 // the same fit, costs 1150 + 165 per warp, and each launch its edge: 2240
 // cycles (1.15 us) in a graph, 0.9 us more outside. Two steps per launch run
@@ -19,7 +19,7 @@ namespace clbm {
 // 1.80 / 2.12 -> 1.31 / 1.45, 16 x 32 x 32 2.08 / 2.67 -> 1.69 / 2.44,
 // 64 x 64 x 5 2.18 / 2.45 -> 1.82 / 2.27, 128 x 128 x 5 3.27 / 4.18 -> 3.23 /
 // 3.16, 32^3 2.32 / 2.89 -> 2.45 / 2.61.
-bool small_plan(const Geom &g, SmallPlan &p) {
+bool small_plan(const Geom &g, int sms, SmallPlan &p) {
     const int64_t n = (int64_t)g.nx * g.ny * g.nz;
     if (g.slab || n >= 100000) return false;
     double best = 1e300;
@@ -43,7 +43,7 @@ bool small_plan(const Geom &g, SmallPlan &p) {
                 const int we = (ext + 31) / 32, wo = (bx * by * bz + 31) / 32;
                 const int resident = std::min({32 / we, 64 / we, (int)(220 * 1024 / (ext * kQ * 4 + 1024))});
                 if (resident < 1) return;
-                const double blocks = (double)nbx * nby * nbz, per_sm = std::ceil(blocks / 152.0);
+                const double blocks = (double)nbx * nby * nbz, per_sm = std::ceil(blocks / sms);
                 if (per_sm > resident) return;
                 const double cost = 2100.0 + per_sm * 190.0 * (we + wo);
                 if (cost < best) {
@@ -57,7 +57,7 @@ bool small_plan(const Geom &g, SmallPlan &p) {
             });
         });
     });
-    const double edge = 2240.0, more = 1750.0, single = 1150.0 + 165.0 * std::ceil((double)n / (152 * 32));
+    const double edge = 2240.0, more = 1750.0, single = 1150.0 + 165.0 * std::ceil((double)n / ((double)sms * 32));
     if (best + edge + more >= 2.0 * (single + edge + more)) return false;
     p.in_graph = best + edge < 2.0 * (single + edge);
     // quotients of thread indices below 1024 by multiplication; a divisor of 1 has no such factor
