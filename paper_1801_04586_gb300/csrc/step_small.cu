@@ -1,7 +1,9 @@
 // step_small.cu -- plan and launch of the two-step kernel of small lattices
 // (step_small.cuh).
 #include <algorithm>
+#include <atomic>
 #include <cmath>
+#include <type_traits>
 
 #include "step_small.cuh"
 
@@ -41,7 +43,7 @@ bool small_plan(const Geom &g, int sms, SmallPlan &p) {
                 const int hz = nbz > 1, ez = bz + 2 * hz, ext = ex * ey * ez;
                 if (ext > 1024) return;
                 const int we = (ext + 31) / 32, wo = (bx * by * bz + 31) / 32;
-                const int resident = std::min({32 / we, 64 / we, (int)(220 * 1024 / (ext * kQ * 4 + 1024))});
+                const int resident = std::min(32 / we, (int)(220 * 1024 / (ext * kQ * 4 + 1024)));
                 if (resident < 1) return;
                 const double blocks = (double)nbx * nby * nbz, per_sm = std::ceil(blocks / sms);
                 if (per_sm > resident) return;
@@ -70,30 +72,41 @@ bool small_plan(const Geom &g, int sms, SmallPlan &p) {
     return true;
 }
 
-template <int FM>
+template <int FM, bool WALLS>
 static cudaError_t small_t(const Launch &L, const SmallPlan &p, const float *src, float *dst, const Rates &r,
                            const ForceArgs &F, float scale2, int *flag) {
-    auto go = [&](auto kern) -> cudaError_t {
-        const size_t smem = (size_t)kQ * p.ext * sizeof(float);
-        if (smem > 48 * 1024) {
-            const cudaError_t e =
-                cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kQ * 1024 * (int)sizeof(float));
+    const size_t smem = (size_t)kQ * p.ext * sizeof(float);
+    if (smem > 48 * 1024) {
+        // the shared-memory opt-in, once per device for this kernel; host threads
+        // may race to set it, which repeats a harmless call
+        static std::atomic<int> opted_in[64] = {};
+        int dev = 0;
+        cudaError_t e = cudaGetDevice(&dev);
+        if (e != cudaSuccess) return e;
+        if (dev >= 64 || !opted_in[dev].load(std::memory_order_relaxed)) {
+            e = cudaFuncSetAttribute(k_step_small2<FM, WALLS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     kQ * 1024 * (int)sizeof(float));
             if (e != cudaSuccess) return e;
+            if (dev < 64) opted_in[dev].store(1, std::memory_order_relaxed);
         }
-        return launch_overlapped(kern, dim3(p.nbx * p.nby * p.nbz), dim3(p.threads), smem, L.stream, L.overlap, src,
-                                 dst, L.g, r, F, scale2, flag, p);
-    };
-    return L.g.walls ? go(k_step_small2<FM, true>) : go(k_step_small2<FM, false>);
+    }
+    return launch_overlapped(k_step_small2<FM, WALLS>, dim3(p.nbx * p.nby * p.nbz), dim3(p.threads), smem, L.stream,
+                             L.overlap, src, dst, L.g, r, F, scale2, flag, p);
 }
 
 cudaError_t launch_step_small2(const Launch &L, const SmallPlan &p, const void *src, void *dst, const Rates &r,
                                const ForceArgs &F, float scale2, int *flag) {
     const float *s = (const float *)src;
     float *d = (float *)dst;
+    auto walls = [&](auto fm) {
+        constexpr int FM = decltype(fm)::value;
+        return L.g.walls ? small_t<FM, true>(L, p, s, d, r, F, scale2, flag)
+                         : small_t<FM, false>(L, p, s, d, r, F, scale2, flag);
+    };
     switch (F.mode) {
-        case kForceUniform: return small_t<kForceUniform>(L, p, s, d, r, F, scale2, flag);
-        case kForceProfileZ: return small_t<kForceProfileZ>(L, p, s, d, r, F, scale2, flag);
-        default: return small_t<kForceField>(L, p, s, d, r, F, scale2, flag);
+        case kForceUniform: return walls(std::integral_constant<int, kForceUniform>{});
+        case kForceProfileZ: return walls(std::integral_constant<int, kForceProfileZ>{});
+        default: return walls(std::integral_constant<int, kForceField>{});
     }
 }
 
