@@ -631,7 +631,9 @@ def run_gb300(args):
     achieved = bytes_per_node * nodes / mean_launch_s / 1e9
     default_case = (args.storage, args.lattice, args.pattern, args.variant, args.model) == (
         "f32", 19, "ab", 0, "cascaded") and not slab and not strong
-    traffic = profiled_traffic() if default_case and side == N_SIDE else None
+    form = lat.step_form()
+    pair_kernel = default_case and form == "two adjacent nodes per thread"
+    traffic = profiled_traffic() if pair_kernel and side == N_SIDE else None
 
     e2e = None
     if not args.no_e2e:
@@ -762,9 +764,7 @@ def run_gb300(args):
             "data": "synthetic",
             "config": {"workload": workload,
                        "nx": nxy, "ny": nxy, "nz": gside if strong else nzl * (ws if slab else 1), "nu": NU, "F0": F0,
-                       "storage": f"{args.storage} {args.pattern.upper()} "
-                                  + ("two adjacent nodes per thread" if default_case else
-                                     "staged in shared memory" if info["staged"] else "one node per thread"),
+                       "storage": f"{args.storage} {args.pattern.upper()} {form}",
                        "block": [info["block_x"], info["block_y"]],
                        "l2": f"inputs larger than L2: {info['buffers']} population buffer(s) of "
                              f"{info['state_bytes'] / 1e9:.2f} GB vs 129 MB L2, no flush",
@@ -773,8 +773,8 @@ def run_gb300(args):
                          "frac": achieved / peak, "traffic": traffic, "peak_kind": peak_kind,
                          "frac_of_nominal": achieved / NOMINAL_HBM_GBS,
                          "algorithmic_bytes_per_launch": bytes_per_node * nodes,
-                         "kernel": "k_step_pair<1,false,true>" if default_case
-                         else f"step kernel, {args.model} collision, {args.storage} storage, D3Q{args.lattice}, "
+                         "kernel": "k_step_pair<1,false,true>" if pair_kernel
+                         else f"step kernel, {form}, {args.model} collision, {args.storage} storage, D3Q{args.lattice}, "
                               f"{args.pattern} pattern" + (", z-slab (faces + interior launches)" if slab else "")},
             "cpu_baseline": cpu,
             "e2e": e2e,

@@ -188,12 +188,12 @@ typedef struct clbm_info {
     int32_t storage;
     int32_t block_x, block_y; /* block shape in use */
     double s2;                /* 1/(3 nu + 1/2) */
-    int32_t nodes_per_thread; /* 2 with variant 2, else 1 (also where variant 0 collides adjacent nodes in pairs) */
+    int32_t nodes_per_thread; /* of the form that block_x and block_y apply to: 2 with variant 2, else 1 (clbm_get_step_form says which form runs) */
     int32_t q;                /* 19 or 27 */
     int32_t pattern;          /* CLBM_PATTERN_AB or CLBM_PATTERN_AA */
     int32_t buffers;          /* population buffers held: 2 (A/B) or 1 (AA) */
     int32_t model;            /* CLBM_MODEL_* */
-    int32_t staged;           /* 1: steps can stage the pulled rows in shared memory (variant 0; small lattices do not, see clbm_params) */
+    int32_t staged;           /* 1: steps can stage the pulled rows in shared memory (variant 0; clbm_get_step_form says whether they do) */
     int32_t slab;             /* halo faces of a z-slab (clbm_params.slab) */
     int64_t face_bytes;       /* z-slab: bytes of one face's 5 populations (5 x nx x ny values), else 0 */
 } clbm_info;
@@ -216,6 +216,16 @@ int clbm_destroy(clbm_ctx *ctx);
 /* Fill *info with the context's sizes, layout and launch choices (see
  * clbm_info). No GPU work. Errors: CLBM_ERR_ARG for a NULL argument. */
 int clbm_get_info(const clbm_ctx *ctx, clbm_info *info);
+
+/* The kernel form that steps of this context run in now. A force field set
+ * later can change it (D3Q27 and misaligned fields are not staged). */
+#define CLBM_FORM_ONE_NODE  0  /* one node per thread */
+#define CLBM_FORM_TWO_NODES 1  /* nodes x and x + block_x per thread (variant 2) */
+#define CLBM_FORM_PAIRS     2  /* two adjacent nodes per thread */
+#define CLBM_FORM_STAGED    3  /* rows staged in shared memory */
+#define CLBM_FORM_TWO_STEPS 4  /* two time steps per launch, one node per thread; an odd step, and graph replays
+                                * where it is not the faster form, take one step per launch */
+int clbm_get_step_form(const clbm_ctx *ctx, int32_t *form);
 
 /* Body force (Sec. II.A, Eqs. 5-6 and 9; a force density). Exactly one force
  * source is active; the latest call wins. Uniform: F is the same at every node

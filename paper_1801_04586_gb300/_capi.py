@@ -29,6 +29,9 @@ WALL_X, WALL_Y, WALL_Z = 1, 2, 4
 SLAB_LO, SLAB_HI = 1, 2
 SLAB_ALL, SLAB_FACES, SLAB_INTERIOR = 0, 1, 2
 INJECT_DROP_COPY = 1
+# what clbm_get_step_form reports (CLBM_FORM_*)
+FORMS = ("one node per thread", "two nodes per thread", "two adjacent nodes per thread", "staged in shared memory",
+         "two steps per launch")
 
 
 class Params(ctypes.Structure):
@@ -79,6 +82,7 @@ SIGNATURES = {
     "clbm_create": [ctypes.POINTER(Params), P, ctypes.POINTER(P)],
     "clbm_destroy": [P],
     "clbm_get_info": [P, ctypes.POINTER(Info)],
+    "clbm_get_step_form": [P, ctypes.POINTER(ctypes.c_int32)],
     "clbm_set_force_uniform": [P, D, D, D],
     "clbm_set_force_profile_z": [P, P],
     "clbm_set_force_field": [P, P],

@@ -516,9 +516,23 @@ int clbm_get_info(const clbm_ctx *c, clbm_info *info) {
     info->pattern = c->aa ? CLBM_PATTERN_AA : CLBM_PATTERN_AB;
     info->buffers = c->aa ? 1 : 2;
     info->model = c->model;
-    info->staged = c->staged && step_staged(c->g, c->elem, c->buf[0], c->q, c->force.mode) ? 1 : 0;
+    info->staged = c->staged && step_staged(c->g, c->elem, c->buf[0], c->q, c->force) ? 1 : 0;
     info->slab = (int32_t)c->g.slab;
     info->face_bytes = c->g.slab ? (int64_t)5 * c->g.nx * c->g.ny * (int64_t)c->elem : 0;
+    return CLBM_OK;
+}
+
+int clbm_get_step_form(const clbm_ctx *c, int32_t *form) {
+    if (!c || !form) return fail(CLBM_ERR_ARG, "clbm_get_step_form: null pointer");
+    // the choices of launch_step, launch_step_aa and launch_step27 (and of clbm_step for two steps per launch)
+    if (c->run_staged && step_staged(c->g, c->elem, c->buf[0], c->q, c->force))
+        *form = CLBM_FORM_STAGED;
+    else if (c->two_step)
+        *form = CLBM_FORM_TWO_STEPS;
+    else if (c->pairs && (!c->aa || c->p.storage == CLBM_STORAGE_F32))
+        *form = CLBM_FORM_PAIRS;
+    else
+        *form = c->packed ? CLBM_FORM_TWO_NODES : CLBM_FORM_ONE_NODE;
     return CLBM_OK;
 }
 

@@ -70,7 +70,7 @@ static cudaError_t step2_force(const Launch &L, const void *src, void *dst, cons
 
 cudaError_t launch_step(int storage, const Launch &L, const void *src, void *dst, const Rates &r,
                         const ForceArgs &F, int *flag, uint32_t key) {
-    if (L.pairs && !(L.staged && step_staged(L.g, storage == 0 ? 4 : 2, src, 19, F.mode)))
+    if (L.pairs && !(L.staged && step_staged(L.g, storage == 0 ? 4 : 2, src, 19, F)))
         return launch_step_pair(storage, L, src, dst, r, F, flag, key);
     if (!L.packed) return launch_step_with<Cascaded>(storage, L, src, dst, r, F, flag, key);
     switch (storage) {
@@ -82,8 +82,8 @@ cudaError_t launch_step(int storage, const Launch &L, const void *src, void *dst
     }
 }
 
-bool step_staged(const Geom &g, size_t elem, const void *src, int q, int force_mode) {
-    return step_staged_for(g, elem, src, q, force_mode);
+bool step_staged(const Geom &g, size_t elem, const void *src, int q, const ForceArgs &F) {
+    return step_staged_for(g, elem, src, q, F);
 }
 
 cudaError_t launch_step_aa(int storage, const Launch &L, void *f, const Rates &r, const ForceArgs &F, int *flag,

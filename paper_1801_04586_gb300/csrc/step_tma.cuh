@@ -155,6 +155,9 @@ inline bool tile_plan(const Geom &g, size_t elem, const void *src, int grid, int
     return true;
 }
 
+// A force field's rows are copied in bulk too: 16-byte aligned component arrays.
+inline bool tile_field_ok(const ForceArgs &F) { return (((uintptr_t)F.field) & 15u) == 0 && (F.n & 3) == 0; }
+
 // ---------------------------------------------------------------- PTX wrappers
 __device__ __forceinline__ uint32_t smem_addr(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -830,7 +833,7 @@ bool launch_step_tma_shape(const Launch &L, const void *src, void *dst, const R 
         if (!tile_plan(L.g, sizeof(S), src, 0, SH::pitch, p, SLAB ? L.z0 : 0, SLAB ? L.zs : 1,
                        SLAB ? L.nplanes : -1))
             return false;
-        if (FM == kForceField && ((((uintptr_t)F.field) & 15u) != 0 || (F.n & 3) != 0)) return false;
+        if (FM == kForceField && !tile_field_ok(F)) return false;
         int dev = 0, sms = 0;
         if ((err = cudaGetDevice(&dev)) != cudaSuccess) return true;
         if ((err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return true;
@@ -894,12 +897,13 @@ bool launch_step_tma(const Launch &L, const void *src, void *dst, const R &r, co
     }
 }
 
-// Whether a step of this context would run staged (for clbm_info).
-inline bool step_staged_for(const Geom &g, size_t elem, const void *src, int q, int force_mode) {
+// Whether a step on this geometry, buffer and force can run staged.
+inline bool step_staged_for(const Geom &g, size_t elem, const void *src, int q, const ForceArgs &F) {
     TilePlan p;
     if (!tile_plan(g, elem, src, 0, 1024, p)) return false;
-    if (q == 27 && force_mode == kForceField) return tile_fits<__half, kForceField, 27, TmaShape27>();
-    return true;
+    if (F.mode != kForceField) return true;
+    if (q == 27 && !tile_fits<__half, kForceField, 27, TmaShape27>()) return false;
+    return tile_field_ok(F);
 }
 
 }  // namespace clbm

@@ -105,6 +105,12 @@ class Lattice:
         check(self.lib.clbm_get_info(self.h, ctypes.byref(i)), "clbm_get_info")
         return {k: getattr(i, k) for k, _ in _capi.Info._fields_}
 
+    def step_form(self) -> str:
+        """The kernel form that steps run in now, one of _capi.FORMS."""
+        f = ctypes.c_int32()
+        check(self.lib.clbm_get_step_form(self.h, ctypes.byref(f)), "clbm_get_step_form")
+        return _capi.FORMS[f.value]
+
     # ---- helpers
     def _dev(self, t: torch.Tensor, shape, name):
         if t.device != self.device or t.dtype != torch.float32 or not t.is_contiguous():
