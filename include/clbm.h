@@ -112,9 +112,8 @@ extern "C" {
  *      and the cascaded D3Q19 in-place (AA) steps with 16-bit storage, stage
  *      the rows they read in shared memory with bulk asynchronous copies
  *      where the geometry allows (nx <= 1024, nx a multiple of 8; D3Q27 not
- *      with a force field) and the lattice is large enough for that to be the
- *      faster form (from 250,000 to 1,500,000 nodes on, see capi.cu; always if
- *      wait_cycles is set); other cascaded D3Q19 A/B steps, and FP32
+ *      with a force field) and that is the faster form for the lattice's size,
+ *      tiles and walls (staged_pays in capi.cu; always if wait_cycles is set); other cascaded D3Q19 A/B steps, and FP32
  *      in-place steps, of lattices of 100,000 nodes or more collide two adjacent nodes per thread
  *      (unless block_x or block_y is given); one node per thread otherwise; 1: always one node per thread,
  *      plain loads (block_x, block_y apply); 2: two nodes per thread (x and

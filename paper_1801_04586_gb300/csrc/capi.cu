@@ -88,7 +88,7 @@ struct clbm_ctx {
     bool packed;          // step kernel with two nodes per thread (FP32x2 arithmetic)
     bool pairs;           // steps with two adjacent nodes per thread where they are not staged (step_pair.cu)
     bool staged;          // steps with rows staged in shared memory by bulk copies apply (variant 0; see clbm_create)
-    bool run_staged;      // ... and the lattice is large enough for them to pay
+    bool run_staged;      // ... and are the faster form (staged_pays)
     int q;                // 19 (Appendix A) or 27 (Sec. II)
     bool aa;              // in-place (AA) pattern: one population buffer, step kind by parity
     int model;            // CLBM_MODEL_*
@@ -177,43 +177,6 @@ Launch step_launch_of(const clbm_ctx *c) {
     return L;
 }
 
-// Whether a lattice's 16-bit steps run staged. The staged blocks work through
-// tiles of up to 1024 nodes, two blocks per SM: a lattice of fewer tiles, or of
-// little more than one round of them, leaves SMs idle or waiting on one tile's
-// copy latency. Measured (us a step, staged / the form that replaces it):
-//   A/B cascaded against node pairs: FP16 48^3 4.9 / 3.0, 80^3 10.3 / 9.2,
-//     104^3 20.4 / 18.0, 112^3 23.4 / 24.8, 128^3 34.4 / 36.9, 256^3 228 / 271;
-//     FP16-SR 48^3 6.8 / 4.3, 104^3 22.4 / 19.0, 112^3 25.6 / 25.0, 128^3 37.3
-//     / 37.9, 256^3 251 / 278; below 100,000 nodes against one node per thread
-//     32^3 6.1 / 2.2;
-//   A/B SRT and MRT against one node: 64^3 6.7 / 5.8, 96^3 17.5 / 15.7, 104^3
-//     with walls 23.0 / 27.2, 112^3 24.8 / 27.7;
-//   in place and D3Q27 against one node, by the share of the rounds' tiles
-//     that are full: in place FP16 56^3 (0.56) 7.0 / 5.2, 64^3 (0.84) 6.7 /
-//     6.3, 80^3 (0.82) 10.9 / 12.6, 64 x 64 x 80 with walls (0.53) 9.7 / 8.4,
-//     104 x 64 x 56 (0.60) 10.2 / 11.2; BF16-SR 64^3 7.4 / 7.5, 72^3 (0.60)
-//     11.9 / 13.0; D3Q27 FP16 56^3 9.2 / 7.4, 64^3 9.2 / 9.1, 72^3 15.0 /
-//     16.3, 64 x 64 x 80 with walls 18.0 / 12.1, 200 x 32 x 40 (0.82) 9.3 /
-//     10.5; FP16-SR 64^3 9.5 / 10.9.
-// A context that bounds or injects the staged waits runs them at any size, as
-// do z-slabs (not measured across GPUs) and the bounds-checked build.
-bool staged_pays(const clbm_params &p, int q, bool pairs) {
-#ifdef CLBM_BOUNDS_CHECK
-    return true;
-#endif
-    if (p.slab || p.inject || p.wait_cycles > 0) return true;
-    const int64_t n = (int64_t)p.nx * p.ny * p.nz;
-    const bool stochastic = p.storage == CLBM_STORAGE_F16_SR || p.storage == CLBM_STORAGE_BF16_SR;
-    if (q == 19 && p.pattern == CLBM_PATTERN_AB) {
-        if (p.model != CLBM_MODEL_CASCADED) return n >= 900000;
-        if (pairs) return n >= (stochastic ? 1500000 : 1200000);
-    }
-    if (n < 250000 || p.nx > 1024) return n >= 250000;
-    const int64_t rows = std::min<int64_t>(p.ny, 1024 / p.nx), tiles = (p.ny + rows - 1) / rows * p.nz;
-    const int64_t rounds = (tiles + 303) / 304;
-    return (double)n >= 0.58 * (double)rounds * 304 * 1024 || n >= 1000000;
-}
-
 // SMs of the current device (1 if that cannot be asked: the allocations that follow then report the error).
 int device_sms() {
     int dev = 0, sms = 0;
@@ -222,6 +185,60 @@ int device_sms() {
         return sms;
     cudaGetLastError();
     return 1;
+}
+
+// Whether a lattice's 16-bit steps run staged. Measured at 0.1 to 16 M nodes,
+// both forms go by simple quantities: a staged step by the rounds of tiles that
+// its resident blocks work through, whether those are full or not, and by some
+// rounds' worth of copy latency before them; the unstaged one by its lanes (one
+// node per thread: idle lanes of partial blocks included; node pairs: the
+// nodes). So a step runs staged if
+//   lanes >= share x (nodes of a round of full tiles) x (rounds + start).
+// share and start are fitted for each family of kernels, rounding to nearest /
+// stochastic, on 180-320 lattices each with nx from 24 to 1024, start by the
+// walls: none, y, z (a z wall's tiles read 5 or 9 of 19 or 27 populations from
+// global memory), x (every tile does; inf: the unstaged step won at every
+// size). The form chosen is the slower one by more than 5 % on 3 % of them,
+// which costs 0.1-0.7 % on average. us a step, staged / unstaged:
+//   in place: FP16 64^3 6.7 / 6.3, 80^3 10.3 / 12.1, 520 x 80 x 64 63.3 / 55.4,
+//     128^3 35.2 / 40.7; FP16-SR with y, z walls 64^3 10.3 / 8.4, 96^3 21.5 / 24.6;
+//   D3Q27: FP16 128 x 64 x 50 12.7 / 13.5, with y, z walls 16.3 / 14.9, with x
+//     walls 256 x 256 x 160 488 / 335; FP16-SR 520 x 20 x 30 11.2 / 13.1;
+//   SRT and MRT: D3Q19 FP16 80^3 11.0 / 11.5, 264 x 60 x 60 with y, z walls 25.9
+//     / 20.8; D3Q27 128^3 51.9 / 55.4, with y, z walls 68.8 / 60.1;
+//   A/B cascaded, staged / pairs: FP16 104^3 20.4 / 18.0, 128^3 34.5 / 36.9, 520
+//     x 256 x 80 225 / 174, 256 x 256 x 160 145 / 171; FP16-SR 128^3 37.5 / 37.8.
+// A context that bounds or injects the staged waits runs them at any size, as
+// do z-slabs (not measured across GPUs) and the bounds-checked build.
+bool staged_pays(const clbm_ctx *c, int sms) {
+#ifdef CLBM_BOUNDS_CHECK
+    return true;
+#endif
+    const clbm_params &p = c->p;
+    if (p.slab || p.inject || p.wait_cycles > 0) return true;
+    struct Line {
+        double share, start[4];  // walls: none, y, z, x
+    };
+    constexpr double inf = 1e30;
+    static const Line lines[5][2] = {
+        {{0.56, {0.5, 0.1, 0.6, 3.3}}, {0.32, {1.7, 2.1, 2.2, 4.1}}},  // cascaded against single D3Q19 nodes (in place)
+        {{0.54, {3.0, 2.4, 2.6, 6.0}}, {0.64, {2.1, 2.4, 2.1, inf}}},  // cascaded against D3Q19 node pairs (A/B)
+        {{0.44, {0.8, 1.0, 4.7, inf}}, {0.30, {1.2, 2.0, 3.2, inf}}},  // cascaded D3Q27
+        {{0.66, {0.9, 0.1, 1.2, inf}}, {0.58, {1.4, 1.3, 2.6, inf}}},  // SRT, MRT
+        {{0.66, {0.2, 0.6, 2.9, inf}}, {0.78, {0.2, 0.5, 3.3, inf}}},  // SRT, MRT D3Q27
+    };
+    const bool cascaded = p.model == CLBM_MODEL_CASCADED;
+    int rounds = 0;
+    int64_t capacity = 0;
+    if (!staged_rounds(c->g, c->q, cascaded, sms, rounds, capacity)) return false;
+    const bool stochastic = p.storage == CLBM_STORAGE_F16_SR || p.storage == CLBM_STORAGE_BF16_SR;
+    const bool against_pairs = c->pairs && !c->aa;
+    const int family = cascaded ? (c->q == 27 ? 2 : against_pairs ? 1 : 0) : (c->q == 27 ? 4 : 3);
+    const Line &l = lines[family][stochastic];
+    const int w = (p.walls & 1u) ? 3 : (p.walls & 4u) ? 2 : (p.walls & 2u) ? 1 : 0;
+    const int64_t bx = c->block.x, by = c->block.y;
+    const int64_t lanes = against_pairs ? c->n : (p.nx + bx - 1) / bx * bx * ((p.ny + by - 1) / by * by) * p.nz;
+    return (double)lanes >= l.share * (double)capacity * (rounds + l.start[w]);
 }
 
 bool rate_ok(double s) { return std::isfinite(s) && s > 0.0 && s < 2.0; }
@@ -426,12 +443,14 @@ int clbm_create(const clbm_params *p, void *stream, clbm_ctx **out) {
     // staged: A/B steps, and the cascaded D3Q19 in-place step (node pairs), where they pay
     c->staged = p->variant == 0 &&
                 (p->pattern != CLBM_PATTERN_AA || (q == 19 && p->model == CLBM_MODEL_CASCADED));
-    c->run_staged = c->staged && staged_pays(*p, q, c->pairs);
     c->aa = p->pattern == CLBM_PATTERN_AA;
     c->model = p->model;
+    c->block = dim3(bx, by, 1);
+    const int sms = device_sms();
+    c->run_staged = c->staged && c->elem == 2 && staged_pays(c, sms);
     c->two_step = q == 19 && p->variant == 0 && p->storage == CLBM_STORAGE_F32 && p->pattern == CLBM_PATTERN_AB &&
                   p->model == CLBM_MODEL_CASCADED && p->block_x == 0 && p->block_y == 0 &&
-                  small_plan(c->g, device_sms(), c->small);
+                  small_plan(c->g, sms, c->small);
     c->rates27.om2 = c->rates.om2;
     c->rates27.cb = c->rates.cb;
     c->rates27.om3 = c->rates.om3;
@@ -442,7 +461,6 @@ int clbm_create(const clbm_params *p, void *stream, clbm_ctx **out) {
     c->rates27.om5 = (float)(1.0 - s5);
     c->rates27.c5 = (float)((1.0 - 0.5 * s5) / 9.0);
     c->rates27.om6 = (float)(1.0 - s6);
-    c->block = dim3(bx, by, 1);
     c->cur = 0;
     c->steps_done = 0;
     const size_t bytes = (state_bytes(c) + 255) / 256 * 256;  // both buffers 256-byte aligned

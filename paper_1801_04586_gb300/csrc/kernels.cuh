@@ -124,6 +124,10 @@ cudaError_t launch_step_slab(int storage, const Launch &L, const void *src, void
 // (elem bytes per value) with force F runs the shared-memory staged kernel
 // (step_tma.cuh) when the launch asks for it.
 bool step_staged(const Geom &g, size_t elem, const void *src, int q, const ForceArgs &F);
+// The rounds of tiles of a 16-bit staged step on a device of sms SMs, and the
+// nodes that a round of full tiles holds; pairs: a collision in node pairs (the
+// cascaded one). False where the geometry is not staged.
+bool staged_rounds(const Geom &g, int q, bool pairs, int sms, int &rounds, int64_t &capacity);
 // In-place (AA) pattern: one step on the single population array f; odd
 // selects the odd step kind (step.cu).
 cudaError_t launch_step_aa(int storage, const Launch &L, void *f, const Rates &r, const ForceArgs &F, int *flag,

@@ -82,6 +82,10 @@ cudaError_t launch_step(int storage, const Launch &L, const void *src, void *dst
     }
 }
 
+bool staged_rounds(const Geom &g, int q, bool pairs, int sms, int &rounds, int64_t &capacity) {
+    return staged_rounds_for(g, q, pairs, sms, rounds, capacity);
+}
+
 bool step_staged(const Geom &g, size_t elem, const void *src, int q, const ForceArgs &F) {
     return step_staged_for(g, elem, src, q, F);
 }

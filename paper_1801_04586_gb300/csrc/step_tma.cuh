@@ -155,6 +155,18 @@ inline bool tile_plan(const Geom &g, size_t elem, const void *src, int grid, int
     return true;
 }
 
+// Blocks of a launch of which `resident` fit the device at once. Block b takes
+// the tiles b, b + grid, ...; with a grid sharing a factor with the tiles per
+// plane a block meets only some row positions, and the few blocks whose
+// positions hold the y-wall rows take all the slower wall tiles. A grid coprime
+// to it spreads them evenly.
+inline int tile_grid(const TilePlan &p, int resident, bool walls) {
+    int grid = p.ntiles < resident ? p.ntiles : resident;
+    if (walls && grid < p.ntiles)
+        while (grid > 1 && std::gcd(grid, p.tiles_y) != 1) --grid;
+    return grid;
+}
+
 // A force field's rows are copied in bulk too: 16-byte aligned component arrays.
 inline bool tile_field_ok(const ForceArgs &F) { return (((uintptr_t)F.field) & 15u) == 0 && (F.n & 3) == 0; }
 
@@ -838,12 +850,7 @@ bool launch_step_tma_shape(const Launch &L, const void *src, void *dst, const R 
         if ((err = cudaGetDevice(&dev)) != cudaSuccess) return true;
         if ((err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return true;
         constexpr size_t smem = tile_smem_bytes<S, FM, Q, SH>();
-        int grid = p.ntiles < SH::blocks * sms ? p.ntiles : SH::blocks * sms;
-        // Block b takes the tiles b, b + grid, ...; with a grid sharing a factor with the tiles per plane a
-        // block meets only some row positions, and the few blocks whose positions hold the y-wall rows take
-        // all the slower wall tiles. A grid coprime to it spreads them evenly.
-        if (WALLS && grid < p.ntiles)
-            while (grid > 1 && std::gcd(grid, p.tiles_y) != 1) --grid;
+        const int grid = tile_grid(p, SH::blocks * sms, WALLS);
         tile_plan(L.g, sizeof(S), src, grid, SH::pitch, p, SLAB ? L.z0 : 0, SLAB ? L.zs : 1, SLAB ? L.nplanes : -1);
         if (L.wait_cycles > 0) p.wait = L.wait_cycles;
         if (L.drop_first_tile) p.drop_tile = 0;
@@ -895,6 +902,23 @@ bool launch_step_tma(const Launch &L, const void *src, void *dst, const R &r, co
         return launch_step_tma_shape<TmaShape19W, true, Q, C, S, FM, MODE>(L, src, dst, r, F, flag, key, err) ||
                launch_step_tma_shape<TmaShape19, true, Q, C, S, FM, MODE>(L, src, dst, r, F, flag, key, err);
     }
+}
+
+// The tiles of a 16-bit staged step: the rounds of them that its blocks work
+// through, and the nodes of a round of full tiles. False if it does not apply.
+inline bool staged_rounds_for(const Geom &g, int q, bool pairs, int sms, int &rounds, int64_t &capacity) {
+    auto with = [&](auto sh) {
+        using SH = decltype(sh);
+        TilePlan p;
+        if (!tile_plan(g, 2, nullptr, 0, SH::pitch, p)) return false;
+        const int grid = tile_grid(p, SH::blocks * sms, g.walls != 0);
+        rounds = (p.ntiles + grid - 1) / grid;
+        capacity = (int64_t)SH::blocks * sms * SH::pitch;
+        return true;
+    };
+    if (q == 27) return pairs ? with(TmaShape27P{}) : with(TmaShape27{});
+    if (pairs) return with(TmaShape19P{});
+    return (g.walls && with(TmaShape19W{})) || with(TmaShape19{});
 }
 
 // Whether a step on this geometry, buffer and force can run staged.

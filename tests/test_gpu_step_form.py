@@ -44,6 +44,27 @@ def test_step_form(shape, kw, form):
     g.close()
 
 
+@pytest.mark.parametrize("shape,kw,form", [
+    # tiles of 520 nodes (one row each, half full) in two full rounds: rounds count, not nodes
+    ((520, 20, 30), dict(storage="f16sr", lattice=27), STAGED),
+    ((600, 25, 24), dict(storage="f16", lattice=27), STAGED),
+    ((520, 80, 64), dict(storage="f16", pattern="aa"), ONE),
+    ((520, 80, 64), dict(storage="f16"), PAIRS),
+    # SRT and MRT below the node pairs' sizes; z walls make whole planes of slow tiles, x walls every tile
+    ((80, 80, 80), dict(storage="f16", model="mrt"), STAGED),
+    ((264, 60, 60), dict(storage="f16", model="mrt", walls=6), ONE),
+    ((128, 128, 128), dict(storage="f16", model="srt", walls=1), ONE),
+    ((128, 128, 100), dict(storage="f16", lattice=27), STAGED),
+    ((128, 128, 100), dict(storage="f16", lattice=27, walls=1), ONE),
+    ((64, 64, 64), dict(storage="f16sr", pattern="aa", walls=6), ONE),
+    ((96, 96, 96), dict(storage="f16sr", pattern="aa", walls=6), STAGED),
+])
+def test_form_follows_the_tiles(shape, kw, form):
+    g = Lattice(*shape, 0.02, device=dev(), **kw)
+    assert g.step_form() == form
+    g.close()
+
+
 def test_step_form_follows_the_force():
     nx, ny, nz = 128, 128, 128
     g = Lattice(nx, ny, nz, 0.02, storage="f16", lattice=27, device=dev())
