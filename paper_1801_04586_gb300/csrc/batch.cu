@@ -393,6 +393,7 @@ Launch domain_launch(const clbm_batch *b, int d) {
     L.block = dim3(bx, by, 1);
     L.grid = dim3((g.nx + bx - 1) / bx, (g.ny + by - 1) / by, g.nz);
     L.stream = b->stream;
+    L.overlap = stream_overlaps(b->stream);
     L.packed = false;
     L.staged = false;  // the per-domain schedule runs the one-node kernels
     // state maps: A/B pull map; in place, natural slots after an even number of steps, the odd map after an odd
@@ -499,7 +500,7 @@ int default_tile(const clbm_batch &b) {
 // One step of every domain: A/B from buffer `from`; in place, the odd kind when
 // `from` is 1 (the parity of the step).
 cudaError_t launch_all(clbm_batch *b, cudaStream_t s, int from) {
-    const bool overlap = s != b->capture_stream;
+    const bool overlap = stream_overlaps(s);
     return with_storage(b->storage, [&](auto v) {
         using S = decltype(v);
         return b->aa ? batch_launch_aa_t<S>(b->form, b->buf[0], b->d_descs, b->ndom, b->d_tiles, b->ntiles,

@@ -155,6 +155,7 @@ Launch launch_of(const clbm_ctx *c) {
     L.block = c->block;
     L.grid = dim3((c->g.nx + c->block.x - 1) / c->block.x, (c->g.ny + c->block.y - 1) / c->block.y, c->g.nz);
     L.stream = c->stream;
+    L.overlap = stream_overlaps(c->stream);
     L.packed = false;
     L.staged = c->run_staged;
     L.pairs = c->pairs;

@@ -23,10 +23,17 @@ __device__ __forceinline__ void grid_dependency_wait() {
 // become resident while its predecessor in the stream drains (programmatic
 // stream serialization) if overlap is set. From kernel to kernel in a stream
 // that takes about 1.5 us instead of 4.1 (144 blocks of 128 threads that move
-// one float each). Launches captured into a graph do without: there a plain
-// edge takes 1.15 us, and early-resident blocks crowd onto the SMs that the
-// running kernel leaves free (the 16 x 32 x 32 channel: 2.7 against 2.2 us a
-// step).
+// one float each). Launches captured into a graph, the library's or a
+// caller's, do without (stream_overlaps): there a plain edge takes 1.15 us, and
+// early-resident blocks crowd onto the SMs that the running kernel leaves free
+// (the 16 x 32 x 32 channel: 2.7 against 2.2 us a step).
+inline bool stream_overlaps(cudaStream_t stream) {
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &st) == cudaSuccess) return st == cudaStreamCaptureStatusNone;
+    cudaGetLastError();  // (the launch itself reports what is wrong with the stream)
+    return false;
+}
+
 template <typename... P, typename... A>
 cudaError_t launch_overlapped(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                               bool overlap, A &&...args) {
@@ -78,7 +85,7 @@ struct Launch {
     Geom g;
     dim3 block, grid;  // grid of the one-node-per-thread kernels
     cudaStream_t stream;
-    bool overlap = true;  // launch_overlapped: not inside a graph capture
+    bool overlap = true;  // launch_overlapped: not inside a graph capture (stream_overlaps)
     bool pairs = false;   // launch_step, where the staged form does not apply: two adjacent nodes per thread (step_pair.cu)
     bool packed;       // launch_step: two nodes per thread (grid.x halved)
     bool staged;       // launch_step (A/B) and launch_step_aa (16-bit, cascaded): rows staged by bulk copies
