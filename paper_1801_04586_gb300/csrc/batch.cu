@@ -178,21 +178,21 @@ __global__ void __launch_bounds__(MAXT, pair_blocks(sizeof(S) == 4) * 128 / MAXT
             const uint32_t row =
                 (ez19(i) > 0 ? zm : (ez19(i) < 0 ? zp : zc)) + (ey19(i) > 0 ? rm : (ey19(i) < 0 ? rp : rc));
             if (ex19(i) > 0)
-                h[i] = mk2(ld_state(base + CLBM_IDX(g, row + xam)), ld_state(base + CLBM_IDX(g, row + (two ? xa : xam))));
+                h[i] = mk2(ld_state(CLBM_AT(g, src, base, row + xam, 0u)), ld_state(CLBM_AT(g, src, base, row + (two ? xa : xam), 0u)));
             else if (ex19(i) < 0)
-                h[i] = mk2(ld_state(base + CLBM_IDX(g, row + (two ? xb : xbp))), ld_state(base + CLBM_IDX(g, row + xbp)));
+                h[i] = mk2(ld_state(CLBM_AT(g, src, base, row + (two ? xb : xbp), 0u)), ld_state(CLBM_AT(g, src, base, row + xbp, 0u)));
             else if (even)
-                h[i] = f2{ld_state2(base + CLBM_IDX(g, row + xa))};
+                h[i] = f2{ld_state2(CLBM_AT(g, src, base, row + xa, 1u))};
             else
-                h[i] = mk2(ld_state(base + CLBM_IDX(g, row + xa)), ld_state(base + CLBM_IDX(g, row + xb)));
+                h[i] = mk2(ld_state(CLBM_AT(g, src, base, row + xa, 0u)), ld_state(CLBM_AT(g, src, base, row + xb, 0u)));
         }
         const WallFaces wa = wall_faces(g, (int)xa, y, z), wb = wall_faces(g, (int)xb, y, z);
         if (wa.any() || wb.any()) {
 #pragma unroll
             for (int i = 1; i < kQ; ++i) {
                 const float *base = src + (size_t)opposite(i) * g.stride;
-                if (wa.bounces(i)) h[i].v.x = ld_state(base + CLBM_IDX(g, self));
-                if (wb.bounces(i)) h[i].v.y = ld_state(base + CLBM_IDX(g, self + (xb - xa)));
+                if (wa.bounces(i)) h[i].v.x = ld_state(CLBM_AT(g, src, base, self, 0u));
+                if (wb.bounces(i)) h[i].v.y = ld_state(CLBM_AT(g, src, base, self + (xb - xa), 0u));
             }
         }
         const f2 drho = collide<false>(h, mk2(D->fx), mk2(D->fy), mk2(D->fz), D->r);
@@ -572,7 +572,7 @@ int clbm_batch_create_pattern(const clbm_domain *doms, int32_t ndomains, int32_t
         D.g.walls = p.walls;
         D.g.stride = (n + 63) / 64 * 64;
 #ifdef CLBM_BOUNDS_CHECK
-        D.g.bc_limit = (uint64_t)kQ * D.g.stride;  // the domain's own arrays (violations redirected, not recorded)
+        D.g.bc_limit = (uint64_t)kQ * D.g.stride;  // the domain's own arrays
 #endif
         D.r.om2 = (float)(1.0 - s2);
         D.r.cb = (float)((p.s2b - s2) / 3.0);
@@ -619,9 +619,12 @@ int clbm_batch_create_pattern(const clbm_domain *doms, int32_t ndomains, int32_t
         delete b;
         return bcuda(e, "clbm_batch_create: stream");
     }
+#ifdef CLBM_BOUNDS_CHECK
+    for (DomainDesc &D : b->descs) D.g.bc = (BoundsRecord *)((char *)b->d_flag + 64);  // the flag block's bytes 64-79
+#endif
     e = cudaMemcpyAsync(b->d_descs, b->descs.data(), sizeof(DomainDesc) * ndomains, cudaMemcpyHostToDevice,
                         b->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(b->d_flag, 0, sizeof(int), b->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(b->d_flag, 0, 128, b->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->buf[0], 0, nbuf * (size_t)off * b->elem, b->stream);
     int rc = e == cudaSuccess ? build_tiles(b, default_tile(*b)) : bcuda(e, "clbm_batch_create");
     if (rc != CLBM_OK) {
@@ -809,9 +812,20 @@ int clbm_batch_check(clbm_batch *b, int clear) {
     if (!b) return bfail(CLBM_ERR_ARG, "clbm_batch_check: null pointer");
     int h = 0;
     cudaError_t e = cudaMemcpyAsync(&h, b->d_flag, sizeof(int), cudaMemcpyDeviceToHost, b->stream);
+#ifdef CLBM_BOUNDS_CHECK
+    BoundsRecord rec = {0ull, 0ull};
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(&rec, (char *)b->d_flag + 64, sizeof(rec), cudaMemcpyDeviceToHost, b->stream);
+#endif
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
-    if (e == cudaSuccess && clear) e = cudaMemsetAsync(b->d_flag, 0, sizeof(int), b->stream);
+    if (e == cudaSuccess && clear) e = cudaMemsetAsync(b->d_flag, 0, 128, b->stream);
     if (e != cudaSuccess) return bcuda(e, "clbm_batch_check");
+#ifdef CLBM_BOUNDS_CHECK
+    if (rec.count)
+        return bfail(CLBM_ERR_BOUNDS, "clbm_batch_check: " + std::to_string(rec.count) +
+                                          " out-of-range indices; the first: kind " + std::to_string(rec.first >> 56) +
+                                          ", index " + std::to_string(rec.first & 0x00ffffffffffffffull));
+#endif
     if (h) return bfail(CLBM_ERR_UNSTABLE, "clbm_batch_check: a node's density left (0.1, 1.9) or became non-finite");
     return CLBM_OK;
 }

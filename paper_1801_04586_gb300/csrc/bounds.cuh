@@ -56,6 +56,10 @@ __device__ __forceinline__ uint64_t bc_slots(BoundsRecord *rec, uint64_t base, u
 // The first slot of a node whose slots run from base to base + last: base if
 // base + last is a state-buffer index of g, else 0 (recorded).
 #define CLBM_SLOTS(g, base, last) ::clbm::bc_slots((g).bc, (uint64_t)(base), (uint64_t)(last), (g).bc_limit)
+// base + off, of which `last` elements after it are accessed too; base points
+// into the state buffer that begins at state.
+#define CLBM_AT(g, state, base, off, last)                                                                \
+    ((state) + ::clbm::bc_slots((g).bc, (uint64_t)((base) - (state)) + (off), (uint64_t)(last), (g).bc_limit))
 // Whether the elements [first, first + count) lie below limit (a bulk copy); records if not.
 #define CLBM_RANGE_OK(g, first, count, limit) \
     ::clbm::bc_range((g).bc, (uint64_t)(first), (uint64_t)(count), (uint64_t)(limit))
@@ -63,6 +67,7 @@ __device__ __forceinline__ uint64_t bc_slots(BoundsRecord *rec, uint64_t base, u
 #define CLBM_IDX(g, idx) (idx)
 #define CLBM_SIDX(g, idx, limit) (idx)
 #define CLBM_SLOTS(g, base, last) (base)
+#define CLBM_AT(g, state, base, off, last) ((base) + (off))
 #define CLBM_RANGE_OK(g, first, count, limit) true
 #endif
 

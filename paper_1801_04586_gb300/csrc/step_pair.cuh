@@ -75,13 +75,13 @@ __global__ void __launch_bounds__(kPairThreads) k_step_pair(const float *src, fl
         const float *base = src + (size_t)i * g.stride;
         const uint32_t row = (ez19(i) > 0 ? zm : (ez19(i) < 0 ? zp : zc)) + (ey19(i) > 0 ? rm : (ey19(i) < 0 ? rp : rc));
         if (ex19(i) == 0 && VEC)
-            h[i] = f2{ld_state2(base + CLBM_IDX(g, row + xa))};
+            h[i] = f2{ld_state2(CLBM_AT(g, src, base, row + xa, 1u))};
         else if (ex19(i) == 0)
-            h[i] = mk2(ld_state(base + CLBM_IDX(g, row + xa)), ld_state(base + CLBM_IDX(g, row + xb)));
+            h[i] = mk2(ld_state(CLBM_AT(g, src, base, row + xa, 0u)), ld_state(CLBM_AT(g, src, base, row + xb, 0u)));
         else if (ex19(i) > 0)
-            h[i] = mk2(ld_state(base + CLBM_IDX(g, row + xam)), ld_state(base + CLBM_IDX(g, row + (two ? xa : xam))));
+            h[i] = mk2(ld_state(CLBM_AT(g, src, base, row + xam, 0u)), ld_state(CLBM_AT(g, src, base, row + (two ? xa : xam), 0u)));
         else
-            h[i] = mk2(ld_state(base + CLBM_IDX(g, row + (two ? xb : xbp))), ld_state(base + CLBM_IDX(g, row + xbp)));
+            h[i] = mk2(ld_state(CLBM_AT(g, src, base, row + (two ? xb : xbp), 0u)), ld_state(CLBM_AT(g, src, base, row + xbp, 0u)));
     }
     if (WALLS) {
         const WallFaces wa = wall_faces(g, (int)xa, y, z), wb = wall_faces(g, (int)xb, y, z);
@@ -89,8 +89,8 @@ __global__ void __launch_bounds__(kPairThreads) k_step_pair(const float *src, fl
 #pragma unroll
             for (int i = 1; i < kQ; ++i) {
                 const float *base = src + (size_t)opposite(i) * g.stride;
-                if (wa.bounces(i)) h[i].v.x = ld_state(base + CLBM_IDX(g, self));
-                if (wb.bounces(i)) h[i].v.y = ld_state(base + CLBM_IDX(g, self + (xb - xa)));
+                if (wa.bounces(i)) h[i].v.x = ld_state(CLBM_AT(g, src, base, self, 0u));
+                if (wb.bounces(i)) h[i].v.y = ld_state(CLBM_AT(g, src, base, self + (xb - xa), 0u));
             }
         }
     }
@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(kPairThreads) k_step_aa_pair_even(float *f, Ge
     const bool two = self + 1u < n;  // (the slot after an odd lattice's last node is padding of the array)
     f2 h[kQ];
 #pragma unroll
-    for (int i = 0; i < kQ; ++i) h[i] = f2{ld_state2(f + (size_t)i * g.stride + CLBM_IDX(g, self))};
+    for (int i = 0; i < kQ; ++i) h[i] = f2{ld_state2(CLBM_AT(g, f, f + (size_t)i * g.stride, self, 1u))};
     const uint32_t last = two ? self + 1u : self, plane = (uint32_t)g.nx * (uint32_t)g.ny;
     const int za = FM == kForceProfileZ ? (int)(self / plane) : 0, zb = FM == kForceProfileZ ? (int)(last / plane) : 0;
     f2 fx, fy, fz;
@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(kPairThreads) k_step_aa_pair_even(float *f, Ge
     if (!(fabsf(drho.v.x) < 0.9f) || (two && !(fabsf(drho.v.y) < 0.9f))) *flag = 1;
 #pragma unroll
     for (int i = 0; i < kQ; ++i) {
-        float *to = f + (size_t)opposite(i) * g.stride + CLBM_IDX(g, self);
+        float *to = CLBM_AT(g, f, f + (size_t)opposite(i) * g.stride, self, two ? 1u : 0u);
         if (two)
             *reinterpret_cast<float2 *>(to) = h[i].v;
         else
@@ -189,20 +189,20 @@ __global__ void __launch_bounds__(kPairThreads) k_step_aa_pair_odd(float *f, Geo
             const uint32_t row =
                 (ez19(i) > 0 ? zm : (ez19(i) < 0 ? zp : zc)) + (ey19(i) > 0 ? rm : (ey19(i) < 0 ? rp : rc));
             if (ex19(i) == 0 && VEC)
-                h[i] = f2{ld_state2(base + CLBM_IDX(g, row + xa))};
+                h[i] = f2{ld_state2(CLBM_AT(g, f, base, row + xa, 1u))};
             else if (ex19(i) == 0)
-                h[i] = mk2(ld_state(base + CLBM_IDX(g, row + xa)), ld_state(base + CLBM_IDX(g, row + xb)));
+                h[i] = mk2(ld_state(CLBM_AT(g, f, base, row + xa, 0u)), ld_state(CLBM_AT(g, f, base, row + xb, 0u)));
             else if (ex19(i) > 0)
-                h[i] = mk2(ld_state(base + CLBM_IDX(g, row + xam)), ld_state(base + CLBM_IDX(g, row + (two ? xa : xam))));
+                h[i] = mk2(ld_state(CLBM_AT(g, f, base, row + xam, 0u)), ld_state(CLBM_AT(g, f, base, row + (two ? xa : xam), 0u)));
             else
-                h[i] = mk2(ld_state(base + CLBM_IDX(g, row + (two ? xb : xbp))), ld_state(base + CLBM_IDX(g, row + xbp)));
+                h[i] = mk2(ld_state(CLBM_AT(g, f, base, row + (two ? xb : xbp), 0u)), ld_state(CLBM_AT(g, f, base, row + xbp, 0u)));
         }
         if (WALLS && any) {
 #pragma unroll
             for (int i = 1; i < kQ; ++i) {
                 const float *base = f + (size_t)i * g.stride;
-                if (wa.bounces(i)) h[i].v.x = ld_state(base + CLBM_IDX(g, self));
-                if (wb.bounces(i)) h[i].v.y = ld_state(base + CLBM_IDX(g, self + (xb - xa)));
+                if (wa.bounces(i)) h[i].v.x = ld_state(CLBM_AT(g, f, base, self, 0u));
+                if (wb.bounces(i)) h[i].v.y = ld_state(CLBM_AT(g, f, base, self + (xb - xa), 0u));
             }
         }
     }
@@ -232,13 +232,13 @@ __global__ void __launch_bounds__(kPairThreads) k_step_aa_pair_odd(float *f, Geo
             bb = wb.bounces(opposite(i));
         }
         if (ex19(i) == 0 && VEC && !(WALLS && any)) {
-            *reinterpret_cast<float2 *>(base + CLBM_IDX(g, row + xa)) = h[i].v;
+            *reinterpret_cast<float2 *>(CLBM_AT(g, f, base, row + xa, 1u)) = h[i].v;
         } else {
-            float *back = f + (size_t)opposite(i) * g.stride + CLBM_IDX(g, self);
+            float *back = CLBM_AT(g, f, f + (size_t)opposite(i) * g.stride, self, two ? 1u : 0u);
             const uint32_t oa = row + (ex19(i) > 0 ? (two ? xb : xbp) : (ex19(i) < 0 ? xam : xa));
             const uint32_t ob = row + (ex19(i) > 0 ? xbp : (ex19(i) < 0 ? xa : xb));
-            *(ba ? back : base + CLBM_IDX(g, oa)) = h[i].v.x;
-            if (two) *(bb ? back + 1 : base + CLBM_IDX(g, ob)) = h[i].v.y;
+            *(ba ? back : CLBM_AT(g, f, base, oa, 0u)) = h[i].v.x;
+            if (two) *(bb ? back + 1 : CLBM_AT(g, f, base, ob, 0u)) = h[i].v.y;
         }
     }
 }
@@ -270,7 +270,7 @@ __device__ __forceinline__ uint32_t pair_load(const S *src, const Geom &g, int x
         const size_t pop = (size_t)i * g.stride;
         const uint32_t row = (ez19(i) > 0 ? zm : (ez19(i) < 0 ? zp : zc)) + (ey19(i) > 0 ? rm : (ey19(i) < 0 ? rp : rc));
         if (ex19(i) == 0 && VEC) {
-            h[i] = f2{ld_state2(src + CLBM_IDX(g, pop + (row + xa)))};
+            h[i] = f2{ld_state2(src + CLBM_SLOTS(g, pop + (row + xa), 1u))};
         } else {
             const uint32_t oa = row + (ex19(i) > 0 ? xam : (ex19(i) < 0 ? (two ? xb : xbp) : xa));
             const uint32_t ob = row + (ex19(i) > 0 ? (two ? xa : xam) : (ex19(i) < 0 ? xbp : xb));
