@@ -505,9 +505,10 @@ __device__ __forceinline__ f1 recip_nr(f1 x) { return f1{recip_nr(x.v)}; }
 
 // Correctly rounded 1/x of both lanes: recip_nr's result r is within an ulp, so
 // one more residual step r + r (1 - x r), its residual exact in the fused
-// multiply-add, rounds to the nearest (Markstein 1990, IBM J. Res. Dev. 34);
-// verified against the division for every density in (0.1, 1.9). Lanes outside
-// the normal range of densities (a state the instability flag reports) divide.
+// multiply-add, rounds to the nearest (Markstein 1990, IBM J. Res. Dev. 34).
+// Lanes outside (2^-4, 2^4), states the instability flag reports, divide: there
+// the steps could leave the normal range. Equal to the division for every FP32
+// bit pattern (tests/test_gpu_recip_exact.py).
 __device__ __forceinline__ f2 recip_exact(f2 x) {
     f2 r = recip_nr(x);
     const f2 e = fmaf(-x, r, mk2(1.0f));
