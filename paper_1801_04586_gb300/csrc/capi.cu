@@ -401,10 +401,12 @@ int clbm_create(const clbm_params *p, void *stream, clbm_ctx **out) {
     if (p->model != CLBM_MODEL_CASCADED && p->variant == 2)
         return fail(CLBM_ERR_ARG, "clbm_create: the SRT and MRT models run one node per thread");
     int bx = p->block_x, by = p->block_y;
-    // D3Q27 in place: 93-112 registers leave an SM some 20 warps, which small blocks in 32 x 4 fill best and keep
-    // filled (us a step, default_block_x's shape / 32 x 4: 224 x 192 x 160 FP32 298.8 / 277.6, FP16 280.1 / 225.3,
-    // FP16-SR 313.6 / 280.5; 208 x 160 x 128 FP16 185.8 / 148.4; 128^3 FP32 84.5 / 85.3, FP16 69.6 / 68.8).
-    if (bx == 0) bx = q == 27 && p->pattern == CLBM_PATTERN_AA && p->ny >= 4 ? 32 : default_block_x(p->nx);
+    if (bx == 0) bx = default_block_x(p->nx);
+    // D3Q27 in place: at 93-112 registers an SM holds some 20 warps, which blocks of 5 to 7 warps fill badly. Rows
+    // that would take those run in 32 x 4 (us a step, row-wide blocks / 32 x 4: 224 x 192 x 160 FP32 298.8 / 277.6,
+    // FP16 280.1 / 225.3, FP16-SR 313.6 / 280.5; 208 x 160 x 128 FP16 185.8 / 148.4; 219 x 22 x 28 FP16 6.8 / 6.2),
+    // the others in default_block_x's shape (36 x 13 x 214 FP32 7.95 / 8.28, 111 x 51 x 118 FP16 25.0 / 25.5).
+    if (p->block_x == 0 && bx > 128 && q == 27 && p->pattern == CLBM_PATTERN_AA && p->ny >= 4) bx = 32;
     if (by == 0) by = std::max(1, std::min(p->ny, 128 / bx));
     if (bx < 32 || bx % 32 != 0 || by < 1 || bx * by > 512)
         return fail(CLBM_ERR_ARG, "clbm_create: block_x must be a multiple of 32 and block_x*block_y <= 512");

@@ -82,19 +82,22 @@ __global__ void __launch_bounds__(256, 4) k_step27(const S *src, S *__restrict__
 // writes population (a,b,c) to the slot the opposite direction was read from.
 // A node writes exactly the slots it read; a slot is read once, by the thread
 // that later overwrites it, so the compiler may order the loads freely.
-// Blocks of 256 that the in-place kernel's registers are held to (0: the
-// compiler's choice). The cascaded FP32 even kind takes 93 registers by itself
-// (20 warps per SM), 80 in 24 warps when held to three blocks; a force field
-// then spills more than that gains, and the odd kind's 80 registers come out
-// faster only under a uniform force without walls. us a step, mean of both
-// kinds, free / held: 224 x 192 x 160 uniform 277.6 / 266.8, with walls 278.4 /
-// 275.0 (odd kind held too: 284.3), z profile 269.3 / 265.5, force field 274.5
-// / 296.6 (left free); 96 x 256 x 200 uniform 198.0 / 191.3.
+// In-place kernels whose registers are held to three blocks of 256 on lattices
+// of kHeldNodes nodes or more. The cascaded FP32 even kind takes 93 registers by
+// itself (20 warps per SM), 80 (8 bytes spilled) in 24 warps when held; a force field then
+// spills more than that gains, and the odd kind's 80 registers come out faster
+// only under a uniform force without walls. us a step, mean of both kinds in
+// blocks of 32 x 4, free / held: 224 x 192 x 160 uniform 277.6 / 266.8, with
+// walls 278.4 / 275.0 (odd kind held too: 284.3), z profile 269.3 / 265.5, force
+// field 274.5 / 296.6 (left free); 96 x 256 x 200 uniform 198.0 / 191.3. A
+// smaller lattice leaves those warps empty and only feels the spills: 20 x 16 x
+// 24 2.08 / 2.19, 117 x 13 x 109 7.95 / 8.09, 236 x 42 x 68 24.0 / 23.7.
 template <typename C, typename S, int FM, bool WALLS, bool ODD>
-constexpr int kAaBlocks = C::kPairs && sizeof(S) == 4 && (ODD ? FM == kForceUniform && !WALLS : FM != kForceField) ? 3 : 0;
+constexpr bool kAaHeld = C::kPairs && sizeof(S) == 4 && (ODD ? FM == kForceUniform && !WALLS : FM != kForceField);
+constexpr int64_t kHeldNodes = 300000;
 
-template <typename C, typename S, int FM, bool WALLS, bool ODD>
-__global__ void __launch_bounds__(256, kAaBlocks<C, S, FM, WALLS, ODD>)
+template <typename C, typename S, int FM, bool WALLS, bool ODD, bool HELD>
+__global__ void __launch_bounds__(256, HELD ? 3 : 0)
     k_step27_aa(S *f, Geom g, Rates27 r, ForceArgs F, int *__restrict__ flag, uint32_t key) {
     grid_dependency_wait();
     int x, y, z;
@@ -198,16 +201,21 @@ cudaError_t launch_step27_with(int storage, const Launch &L, const void *src, vo
 template <typename C>
 cudaError_t launch_step27_aa_with(int storage, const Launch &L, void *f, const Rates27 &r, const ForceArgs &F,
                                   int *flag, uint32_t key, bool odd) {
+    const bool large = (int64_t)L.g.nx * L.g.ny * L.g.nz >= kHeldNodes;
     CLBM_Q27_STORE(storage, CLBM_Q27_FM(F.mode, {
+        auto go = [&](auto walls, auto odd_kind) {
+            constexpr bool W = decltype(walls)::value, O = decltype(odd_kind)::value;
+            auto kern = k_step27_aa<C, S, FM, W, O, false>;
+            if constexpr (kAaHeld<C, S, FM, W, O>)
+                if (large) kern = k_step27_aa<C, S, FM, W, O, true>;
+            launch_overlapped(kern, L.grid, L.block, 0, L.stream, L.overlap, (S *)f, L.g, r, F, flag, key);
+        };
         if (!odd)
-            launch_overlapped(k_step27_aa<C, S, FM, false, false>, L.grid, L.block, 0, L.stream, L.overlap, (S *)f,
-                              L.g, r, F, flag, key);
+            go(std::false_type{}, std::false_type{});
         else if (L.g.walls)
-            launch_overlapped(k_step27_aa<C, S, FM, true, true>, L.grid, L.block, 0, L.stream, L.overlap, (S *)f,
-                              L.g, r, F, flag, key);
+            go(std::true_type{}, std::true_type{});
         else
-            launch_overlapped(k_step27_aa<C, S, FM, false, true>, L.grid, L.block, 0, L.stream, L.overlap, (S *)f,
-                              L.g, r, F, flag, key);
+            go(std::false_type{}, std::true_type{});
     }))
     return cudaGetLastError();
 }
