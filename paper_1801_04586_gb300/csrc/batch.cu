@@ -218,7 +218,9 @@ __global__ void __launch_bounds__(MAXT, pair_blocks(sizeof(S) == 4) * 128 / MAXT
 // domain table and collision as k_batch_step, so the batch stores the bits of
 // the A/B batch and of each domain stepped alone.
 // The even kind with FP32 wants 84 registers: capped at two blocks of 512 (64)
-// an in-place step of the benchmark's 64 domains takes 1005 instead of 1088 us.
+// an in-place step of the benchmark's 64 domains takes 946 instead of 977 us
+// (tile of 128; with a table too large for shared memory the cap spills 24
+// bytes, 390 us for 600 small domains either way).
 template <typename S, bool SMEM, bool ODD>
 __global__ void __launch_bounds__(512, ODD || sizeof(S) == 2 ? 0 : 2) k_batch_step_aa(S *A, const DomainDesc *__restrict__ doms, int ndom,
                                                        const int4 *__restrict__ tiles, int ntiles,

@@ -9,7 +9,7 @@ namespace clbm {
 // 2.59, 32^3 2.34 / 2.71, 128 x 128 x 5 3.36 / 3.30 and
 // 4.13 / 4.18 launched one by one, 48^3 4.06 / 3.36, 64^3
 // 6.27 / 5.41, 80^3 13.5 / 9.2, 150 x 91 x 61 with a force field 22.5 / 20.6,
-// 200 x 180 x 160 137 / 128, 256^3 371 / 362).
+// 200 x 180 x 160 137 / 128, 256^3 379 / 369).
 bool step_pairs(const Geom &g) {
     const int64_t npx = (g.nx + 1) / 2;
     // the row of a pair by one multiplication: exact while pairs of a plane x pairs of a row < 2^32

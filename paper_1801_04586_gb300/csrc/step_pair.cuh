@@ -8,13 +8,13 @@
 // results are the same bits), forms each address once for two nodes and moves
 // 9 of 19 populations by 64-bit loads and all of them by 64-bit stores. 78-80
 // registers for the pair (96 and 88 with odd rows) keep six blocks of 128, 24
-// warps of pairs, in flight on an SM. 256^3: 362 us a step
-// against 371 (7.05 TB/s algorithmic, 1.04 of the copy rate); 80^3 in L2: 9.2
-// against 13.5.
+// warps of pairs, in flight on an SM. 256^3: 368.6 us a
+// step against 379.2 (6.92 TB/s algorithmic, 1.03 of the copy rate), on other
+// days 361 against 371; 80^3 in L2: 9.2 against 13.5.
 //
 // (A pass of two steps over a column kept in shared memory, which halves the
 // DRAM traffic, measured 38-45k MLUPS in six forms, no more than the single
-// step's 46.4k: 16 warps per SM do not hide its phases.)
+// step's 45.5-46.4k: 16 warps per SM do not hide its phases.)
 #pragma once
 
 #include "cascaded.cuh"
