@@ -494,7 +494,7 @@ typedef struct clbm_domain {
 
 typedef struct clbm_batch_info {
     int32_t ndomains;
-    int32_t ntiles, grid, threads, graph_steps;
+    int32_t ntiles, grid, threads, graph_steps; /* grid: blocks of a step (in place: of the even kind) */
     int64_t total_nodes;
     int64_t state_bytes;   /* both buffers: 2 x state_bytes are allocated */
     int64_t steps_done;
@@ -524,8 +524,9 @@ int clbm_batch_create_pattern(const clbm_domain *domains, int32_t ndomains, int3
                               void *stream, clbm_batch **out);
 int clbm_batch_destroy(clbm_batch *b);
 int clbm_batch_get_info(const clbm_batch *b, clbm_batch_info *info);
-/* Rebuild the work list for another block size (threads per block and
- * nodes per tile: a multiple of 32 in [32, 512]). Synchronises the stream. */
+/* Rebuild the work list for another block size (threads per block; a tile is
+ * as many nodes, or pairs of adjacent nodes where the batch's size makes them
+ * the faster form: a multiple of 32 in [32, 512]). Synchronises the stream. */
 int clbm_batch_set_tile(clbm_batch *b, int32_t threads);
 /* Time trial_steps launches for each block size in {64, 128, 192, 256, 384,
  * 512} (trials read the current state and write the other buffer, so the

@@ -10,7 +10,8 @@
 // (T = threads per block), so every lane has a node whatever the domain's
 // extents, a warp reads contiguous memory, and only a domain's last tile is
 // partial. One block takes one tile, or a grid of (SMs x resident blocks) walks
-// the list with a stride (form_for): one launch covers all domains. Steps are replayed from a captured CUDA graph.
+// the list with a stride (form_for): one launch covers all domains. Steps are
+// replayed from a captured CUDA graph.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -418,7 +419,8 @@ void *domain_ptr(const clbm_batch *b, int which, int d) {
     return (char *)b->buf[which] + (size_t)b->descs[d].offset * b->elem;
 }
 
-// The form a batch of `nodes` nodes steps in with tiles of T threads, us a step of batches of channels and ducts:
+// The form a batch steps in with tiles of T threads (us a step of batches of
+// channels and ducts):
 // A/B, by size (nodes): below 1.2 rounds of resident pair blocks (FP32 280,000,
 //   16-bit 233,000) one node per thread: half as many warps of pairs leave
 //   schedulers idle (T = 128, one node / pairs: FP16 45k 2.97 / 3.49, 94k 4.14
